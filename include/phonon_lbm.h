@@ -122,13 +122,18 @@ typedef enum {
 
 /* Which stream-collide kernel lbm_step launches. */
 typedef enum {
-    LBM_KERNEL_AUTO = 0,     /* up to 16384 nodes: resident for LBM_FP32,     */
-                             /* scalar for LBM_FP64; from 2^24 nodes (nx >=   */
-                             /* 256) wave where it applies (FP32: 5 steps     */
-                             /* per launch, 128-row segments; 16-bit: 4 and   */
-                             /* 256); else                                    */
-                             /* vector when nx allows, else scalar            */
-                             /* (lbm_autotune times the candidates)           */
+    LBM_KERNEL_AUTO = 0,     /* LBM_FP32 up to 5120 nodes (8192 with sides):  */
+                             /* resident; LBM_FP64 up to 16384: scalar; from  */
+                             /* 2^24 nodes (nx >= 256) wave where it applies  */
+                             /* (FP32: 5 steps per launch, 128-row segments;  */
+                             /* 16-bit: 4 and 256); else vector when nx       */
+                             /* allows, else scalar, and LBM_FP32 lattices in */
+                             /* between then take the plain steps of a call   */
+                             /* several per launch (tiles of the lattice held */
+                             /* in registers, or the strips of the wave       */
+                             /* kernel; same results bit for bit), single     */
+                             /* steps only at its end (lbm_autotune times the */
+                             /* candidates)                                   */
     LBM_KERNEL_SCALAR = 1,   /* one thread per node; any nx                   */
     LBM_KERNEL_VECTOR = 2,   /* 16-byte vectors along x; nx % (16/size) == 0  */
     LBM_KERNEL_STAGED = 3,   /* bulk asynchronous copies (TMA engine) of row  */
@@ -277,7 +282,8 @@ long lbm_step_count(const lbm_ctx *ctx);
  * kernel cannot run this lattice (e.g. VECTOR with a ragged nx). */
 lbm_status lbm_set_kernel(lbm_ctx *ctx, int kernel);
 
-/* The kernel lbm_step will launch (never LBM_KERNEL_AUTO). */
+/* The kernel lbm_step will launch (never LBM_KERNEL_AUTO); for a lattice whose
+ * plain steps run several per launch by its size, that of its single steps. */
 int lbm_get_kernel(const lbm_ctx *ctx);
 
 /* Rounding of 16-bit storage (FP16 / BF16 deviations; no counterpart in the
@@ -367,7 +373,7 @@ lbm_status lbm_get_wave_config(const lbm_ctx *ctx, int *steps, int *rows);
  * in milliseconds, the number of launches and the time steps they advanced
  * since timing was turned on (outputs may be NULL): */
 typedef enum {
-    LBM_TIMED_WAVE = 0,      /* multi-step launches (LBM_KERNEL_WAVE)          */
+    LBM_TIMED_WAVE = 0,      /* multi-step launches (wave kernel, tiles)       */
     LBM_TIMED_SINGLE = 1,    /* single-step launches                           */
     LBM_TIMED_RESIDUAL = 2   /* the step of lbm_step_residual (with its sums)  */
 } lbm_timed;

@@ -15,6 +15,8 @@
 
 using namespace plbm;
 
+enum { MULTI_NONE = 0, MULTI_TILE = 1, MULTI_WAVE = 2 };
+
 struct lbm_ctx {
     int device = 0;
     int nx = 0, ny = 0;
@@ -43,6 +45,11 @@ struct lbm_ctx {
     int cluster_req = 0;
     int wave_steps = 4;         // multi-step kernel: steps per launch
     int wave_rows = 128;        // and rows per strip segment
+    // multi-step launches of lattices whose single steps run on `kernel`
+    // (mid sizes, chosen by size or by lbm_autotune)
+    int multi = MULTI_NONE;
+    TilePlan tile;
+    WavePlan wplan;
     int graph_chunk = 64;
     // launch timing (lbm_set_launch_timing): event pairs around launches
     bool timing = false;
@@ -341,7 +348,11 @@ lbm_status finish_residual(lbm_ctx *c, const double (&sums)[5], double *r,
     return LBM_OK;
 }
 
-constexpr long long RESIDENT_AUTO_NODES = 16384;
+// untimed choice: FP32 lattices up to this many nodes run cluster-resident (with
+// sides the tile kernel's extra halo work moves the line up), FP64 ones up to
+// SCALAR_AUTO_NODES one node per thread
+constexpr long long RESIDENT_AUTO_NODES = 5120, RESIDENT_AUTO_NODES_SIDES = 8192;
+constexpr long long SCALAR_AUTO_NODES = 16384;
 constexpr long long WAVE_AUTO_NODES = 1LL << 24;
 
 // Works out the cluster-resident plan (FP32 lattices whose two buffers fit
@@ -363,15 +374,18 @@ int resolve_kernel(lbm_ctx *c, int requested) {
     if (vec_ok && has_tile_refs(c->precision) && prepare_pipe16(c->precision) != cudaSuccess)
         (void)cudaGetLastError();
     // without timing: small FP32 lattices run cluster-resident, n steps per
-    // launch (measured 1.5-2.4x faster than one launch per step up to 16384
-    // nodes; beyond that 16 SMs do less than the whole GPU)
+    // launch; beyond about 5000 nodes the tile kernel on the whole GPU does
+    // more than 16 SMs (128 x 32 channel 0.64 against 0.70 us per step with
+    // tiles, 160 x 40 0.80 / 0.71, 4096 x 4 1.24 / 0.58; squares with sides
+    // 81 x 81 1.01 / 1.12, 101 x 101 1.25 / 1.14)
     if (requested == KERNEL_AUTO && c->precision == PREC_FP32 &&
-        c->plane <= RESIDENT_AUTO_NODES && resident_ok(c))
+        c->plane <= (has_sides(c) ? RESIDENT_AUTO_NODES_SIDES : RESIDENT_AUTO_NODES) &&
+        resident_ok(c))
         return KERNEL_RESIDENT;
     // small FP64 lattices: FP64 arithmetic bounds the step, and one node per
     // thread spreads it over twice the SMs of the 2-node vectors (128 x 32:
     // 5.3-5.6 against 6.2 us per step)
-    if (requested == KERNEL_AUTO && c->precision == PREC_FP64 && c->plane <= RESIDENT_AUTO_NODES)
+    if (requested == KERNEL_AUTO && c->precision == PREC_FP64 && c->plane <= SCALAR_AUTO_NODES)
         return KERNEL_SCALAR;
     if (requested == KERNEL_WAVE) {
         if (!wave_supported(c->precision, c->nx, c->ny, c->bc_x, c->bc_y)) return -1;
@@ -419,6 +433,42 @@ int resolve_kernel(lbm_ctx *c, int requested) {
     if (requested == KERNEL_STAGED && !staged_ok) return -1;
     if (requested == KERNEL_RESIDENT && !resident_ok(c)) return -1;
     return requested;
+}
+
+// The multi-step kernel that a lattice between the cluster-resident and the
+// strip-march sizes runs its plain steps on (FP32): the one of the lesser
+// estimated time per step, where that is less than a launch per step costs.
+// Measured per step against the single-step kernel: 130 x 130 channel tile
+// 0.77 against 3.98 us, 201 x 201 square 1.13 / 4.2, 1024 x 256 channel 1.60
+// / 3.6, 1024^2 4.5 (wave) / 8.3, 2048^2 13.0 (wave) / 44, 2001^2 square 29.8
+// / 81.8; a single step costs 2.2-3.7 us plus about 6 us per 2^20 nodes in
+// L2 (10.5 beyond it).
+void plan_multi(lbm_ctx *c, int requested) {
+    c->multi = MULTI_NONE;
+    if (requested != KERNEL_AUTO || c->precision != PREC_FP32 ||
+        (c->kernel != KERNEL_VECTOR && c->kernel != KERNEL_SCALAR))
+        return;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
+        sms < 1) {
+        (void)cudaGetLastError();
+        return;
+    }
+    double best = (c->kernel == KERNEL_VECTOR ? 2.2 : 3.6) + 5.7e-6 * (double)c->plane;
+    TilePlan tp;
+    const double tile_us = tile_plan(c->nx, c->ny, c->bc_x, c->bc_y, sms, &tp);
+    if (tp.steps > 0 && tile_us < 0.9 * best) {
+        c->multi = MULTI_TILE;
+        c->tile = tp;
+        best = tile_us;
+    }
+    if (!wave_supported(c->precision, c->nx, c->ny, c->bc_x, c->bc_y)) return;
+    WavePlan wp;
+    const double wave_us = wave_plan(c->nx, c->ny, sms, &wp);
+    if (wave_us < best) {
+        c->multi = MULTI_WAVE;
+        c->wplan = wp;
+    }
 }
 
 lbm_status create_common(lbm_grid g, double tau_N, double tau_R, lbm_boundary bc,
@@ -512,6 +562,7 @@ lbm_status create_common(lbm_grid g, double tau_N, double tau_R, lbm_boundary bc
         return s;
     }
     c->kernel = resolve_kernel(c, KERNEL_AUTO);
+    plan_multi(c, KERNEL_AUTO);
     *out = c;
     return LBM_OK;
 }
@@ -562,6 +613,17 @@ cudaError_t wave_launch(const lbm_ctx *c, int src, int steps, cudaStream_t s) {
                                 c->wave_rows, s);
     return launch_step_wave16(c->precision, steps, c->buf[src], c->buf[1 - src], c->nx, c->ny,
                               c->bc_x, c->bc_y, make_coef<float>(c), c->wave_rows, s);
+}
+
+// One launch of `steps` steps of the context's mid-size multi-step kernel
+// (FP32) from buffer src.
+cudaError_t multi_launch(const lbm_ctx *c, int src, int steps, cudaStream_t s) {
+    const float *in = (const float *)c->buf[src];
+    float *out = (float *)c->buf[1 - src];
+    const Coef<float> k = make_coef<float>(c);
+    if (c->multi == MULTI_TILE)
+        return launch_tile(c->tile, steps, in, out, c->nx, c->ny, c->bc_x, c->bc_y, k, s);
+    return launch_step_wave(steps, in, out, c->nx, c->ny, c->bc_x, c->bc_y, k, c->wplan.rows, s);
 }
 
 // Launches in one captured graph of multi-step launches: an even number (the
@@ -676,6 +738,27 @@ lbm_status advance(lbm_ctx *c, long n, bool end_readable) {
         c->cur = last;
         c->n += n;
         c->launches += 1;
+        return LBM_OK;
+    }
+    if (c->multi != MULTI_NONE) {
+        // launched directly: a launch takes longer than its submission, and a
+        // captured graph would have to be built again after every lbm_init
+        const long tail = end_readable ? 1 : 0;
+        const int K = c->multi == MULTI_TILE ? c->tile.steps : c->wplan.steps;
+        long m = n - tail;
+        while (m >= (c->multi == MULTI_TILE ? 1 : WAVE_MIN_STEPS)) {
+            const int k = m >= K ? K : (int)m;
+            int slot;
+            CK(c, timed_begin(c, TIMED_WAVE, k, &slot));
+            CK(c, multi_launch(c, c->cur, k, c->stream));
+            CK(c, timed_end(c, slot));
+            c->cur = 1 - c->cur;
+            m -= k;
+            c->n += k;
+            c->launches += 1;
+        }
+        for (long i = 0; i < m + tail; ++i)
+            if (lbm_status s = single_step(c)) return s;
         return LBM_OK;
     }
     if (c->kernel == KERNEL_WAVE) {
@@ -987,6 +1070,7 @@ lbm_status lbm_set_kernel(lbm_ctx *c, int kernel) {
         drop_graphs(c);
         c->kernel = k;
     }
+    plan_multi(c, kernel);
     return LBM_OK;
 }
 
@@ -1092,8 +1176,10 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
     if (trial_steps & 1) ++trial_steps;       // even: the buffers end where they began
     DeviceGuard g(c->device);
     if (lbm_status s = ensure_scratch(c, false)) return s;   // the status word
-    struct Cand { int kernel, stages, cw; };   // wave: stages = steps, cw = segment rows
-    Cand cands[16];
+    // wave: stages = steps, cw = segment rows; multi: the mid-size multi-step
+    // kernel the lattice's size picks, its single steps on `kernel`
+    struct Cand { int kernel, stages, cw, multi; };
+    Cand cands[17];
     int nc = 0;
     const bool sides = has_sides(c);      // the per-side rules: scalar and vector kernels
     if (c->nx % vector_width(c->precision) == 0) cands[nc++] = {KERNEL_VECTOR, 0, 0};
@@ -1112,6 +1198,17 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
                 for (int rows : {128, 256}) cands[nc++] = {KERNEL_WAVE, ks, rows};
         }
     }
+
+    for (int i = 0; i < nc; ++i) cands[i].multi = MULTI_NONE;
+    const int old_multi = c->multi;
+    if (cands[0].kernel == KERNEL_VECTOR || cands[0].kernel == KERNEL_SCALAR) {
+        const int k0 = c->kernel;
+        c->kernel = cands[0].kernel;
+        plan_multi(c, KERNEL_AUTO);
+        c->kernel = k0;
+        if (c->multi != MULTI_NONE) cands[nc++] = {cands[0].kernel, 0, 0, c->multi};
+    }
+    const int tuned_multi = c->multi;
 
     // keep the state: copy both buffers aside when the lattice holds one
     void *saved = nullptr;
@@ -1140,7 +1237,17 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
         c->kernel = cands[i].kernel;
         c->plan = p;
         long steps_timed = trial_steps;
-        if (c->kernel == KERNEL_WAVE) {
+        if (cands[i].multi != MULTI_NONE) {
+            const int K = tuned_multi == MULTI_TILE ? c->tile.steps : c->wplan.steps;
+            int launches = (trial_steps + K - 1) / K;
+            launches += launches & 1;
+            steps_timed = (long)launches * K;
+            for (int s = 0; s < 2 && err == cudaSuccess; ++s)      // warm-up
+                err = multi_launch(c, s & 1, K, c->stream);
+            if (err == cudaSuccess) err = cudaEventRecord(e0, c->stream);
+            for (int s = 0; s < launches && err == cudaSuccess; ++s)
+                err = multi_launch(c, s & 1, K, c->stream);
+        } else if (c->kernel == KERNEL_WAVE) {
             // its point is several steps per launch: time whole launches, an
             // even number (the buffers end where they began)
             c->wave_steps = cands[i].stages;
@@ -1195,6 +1302,7 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
     if (err != cudaSuccess || best_i < 0) {
         c->kernel = old_kernel;
         c->plan = old_plan;
+        c->multi = old_multi;
         c->wave_steps = old_ws;
         c->wave_rows = old_wr;
         return err != cudaSuccess ? cuda_fail(c, err, "lbm_autotune")
@@ -1204,6 +1312,7 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
     drop_graphs(c);
     c->kernel = cands[best_i].kernel;
     c->plan = best_plan;
+    c->multi = cands[best_i].multi;
     if (cands[best_i].kernel == KERNEL_WAVE) {
         c->wave_steps = cands[best_i].stages;
         c->wave_rows = cands[best_i].cw;

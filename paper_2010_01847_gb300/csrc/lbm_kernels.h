@@ -154,6 +154,12 @@ cudaError_t launch_resident(const float *src, float *out_last, float *out_prev, 
 constexpr int WAVE_MIN_STEPS = 2;
 constexpr int WAVE_MAX_STEPS = 8;
 constexpr int WAVE16_MAX_STEPS = 4;     // 16-bit storage (wave16.cu)
+// Steps per launch and segment rows of the FP32 march for a lattice it takes
+// on a GPU of `sms` SMs, and the estimated time per step in us.
+struct WavePlan {
+    int steps = 0, rows = 0;
+};
+double wave_plan(int nx, int ny, int sms, WavePlan *out);
 bool wave_supported(int precision, int nx, int ny, int bc_x, int bc_y);
 int wave_max_steps(int precision);
 cudaError_t launch_step_wave(int steps, const float *src, float *dst, int nx, int ny, int bc_x,
@@ -164,6 +170,38 @@ cudaError_t launch_step_wave(int steps, const float *src, float *dst, int nx, in
 cudaError_t launch_step_wave16(int precision, int steps, const void *src, void *dst, int nx,
                                int ny, int bc_x, int bc_y, const Coef<float> &k, int seg_rows,
                                cudaStream_t stream);
+// The tile kernel (tile.cu): `steps` time steps in one launch on tiles held
+// in registers, FP32 storage, any nx, ny and boundary kind, results
+// bit-identical to single steps; like the multi-step kernel it keeps the
+// post-collision state of the last step only.
+constexpr int TILE_MAX_WARPS = 16;
+constexpr int TILE_MAX_STEPS = 16;        // tiles of at least 32 own columns
+constexpr int TILE_MAX_ROWS = 4;
+constexpr long long TILE_MAX_NODES = 1LL << 28;     // 32-bit block counts and node columns
+struct TilePlan {
+    int ty = 0;             // own rows of a tile (own columns: 64 less two halos)
+    int rows = 0;           // rows per warp, 1..TILE_MAX_ROWS
+    int steps = 0;          // most steps per launch (0: no plan)
+};
+// Rows a block of a tile of ty own rows holds at most (open: the lattice is
+// bounded by walls or sides along y).
+inline int tile_rows(int ty, int ny, bool open, int steps) {
+    const int own = ty < ny ? ty : ny;
+    return open ? (own + 2 * steps < ny ? own + 2 * steps : ny) : own + 2 * steps;
+}
+// Halo columns of a plan's tiles (even: pairs stay 8-byte aligned) and tiles
+// across nx columns; the tiles at x sides (open) own one halo more.
+inline int tile_halo(int steps) { return (steps + 1) & ~1; }
+inline int tile_columns(const TilePlan &p, int nx, bool open) {
+    const int hx = tile_halo(p.steps), own = 64 - 2 * hx, n = open ? nx - 2 * hx : nx;
+    return n <= own ? 1 : (n + own - 1) / own;
+}
+// The plan for a lattice on a GPU of `sms` SMs and its estimated time per
+// step in us (out->steps = 0: none).
+double tile_plan(int nx, int ny, int bc_x, int bc_y, int sms, TilePlan *out);
+cudaError_t launch_tile(const TilePlan &p, int steps, const float *src, float *dst, int nx, int ny,
+                        int bc_x, int bc_y, const Coef<float> &k, cudaStream_t stream);
+
 // Runs the staged kernel's bounded mbarrier wait against a barrier nothing
 // completes (one CTA, ~2 s); the wait gives up and ORs 1 into *status.
 cudaError_t launch_wait_probe(int *status, cudaStream_t stream);
