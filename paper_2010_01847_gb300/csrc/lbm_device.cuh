@@ -140,7 +140,7 @@ template <> __device__ __forceinline__ float2 splat<float2>(float c) { return ma
 // formed in one rounding (fused multiply-add) and t_i = +t (plus) or -t
 // (minus); t carries the flux factor 1 - zeta, which holds the resistive
 // term sigma t_i of Eq. 16.  For minus the negated equilibrium
-// -eq = w (-rho) + t is formed instead (rounding is symmetric, so it is
+// -eq = (-w) rho + t is formed instead (rounding is symmetric, so it is
 // exactly -eq) and added.
 template <typename V>
 __device__ __forceinline__ V relax_plus(V d, V w, V rho, V t, V neg_omega) {
@@ -148,8 +148,8 @@ __device__ __forceinline__ V relax_plus(V d, V w, V rho, V t, V neg_omega) {
     return f_fma(neg_omega, f_sub(d, eq), d);
 }
 template <typename V>
-__device__ __forceinline__ V relax_minus(V d, V w, V neg_rho, V t, V neg_omega) {
-    const V neg_eq = f_fma(w, neg_rho, t);
+__device__ __forceinline__ V relax_minus(V d, V neg_w, V rho, V t, V neg_omega) {
+    const V neg_eq = f_fma(neg_w, rho, t);
     return f_fma(neg_omega, f_add(d, neg_eq), d);
 }
 
@@ -167,14 +167,18 @@ __device__ __forceinline__ void moments_f32(const V (&d)[8], V &rho, V &mx, V &m
     my = f_sub(f_add(f_sub(d[1], d[3]), s46), s75);
 }
 
-// The relaxation of collide_f32 given the node's moments.
-template <typename V>
+// The relaxation of collide_f32 given the node's moments.  NEGW = false forms
+// -rho once instead of holding the negated weights (the same bits): fewer
+// registers, for the pipelined 16-bit step, which has none to spare (0.4 %
+// slower with them).
+template <typename V, bool NEGW = true>
 __device__ __forceinline__ void relax_f32(V (&d)[8], V rho, V mx, V my, const Coef<float> &k) {
     const V neg_zeta = splat<V>(-k.zeta);
     const V qx = f_fma(neg_zeta, mx, mx);               // (1 - zeta) m
     const V qy = f_fma(neg_zeta, my, my);
-    const V neg_rho = f_mul(splat<V>(-1.f), rho);       // exact
     const V wa = splat<V>(k.w_axis), wd = splat<V>(k.w_diag);
+    const V na = NEGW ? splat<V>(-k.w_axis) : wa, nd = NEGW ? splat<V>(-k.w_diag) : wd;
+    const V nrho = NEGW ? rho : f_mul(splat<V>(-1.f), rho);      // exact
     const V ha = splat<V>(k.h_axis), hd = splat<V>(k.h_diag);
     const V ta = f_mul(ha, qx);
     const V tb = f_mul(ha, qy);
@@ -184,21 +188,23 @@ __device__ __forceinline__ void relax_f32(V (&d)[8], V rho, V mx, V my, const Co
     // t_i for i = 0..7: ta, tb, -ta, -tb, tp, -tm, -tp, tm
     d[0] = relax_plus(d[0], wa, rho, ta, no);
     d[1] = relax_plus(d[1], wa, rho, tb, no);
-    d[2] = relax_minus(d[2], wa, neg_rho, ta, no);
-    d[3] = relax_minus(d[3], wa, neg_rho, tb, no);
+    d[2] = relax_minus(d[2], na, nrho, ta, no);
+    d[3] = relax_minus(d[3], na, nrho, tb, no);
     d[4] = relax_plus(d[4], wd, rho, tp, no);
-    d[5] = relax_minus(d[5], wd, neg_rho, tm, no);
-    d[6] = relax_minus(d[6], wd, neg_rho, tp, no);
+    d[5] = relax_minus(d[5], nd, nrho, tm, no);
+    d[6] = relax_minus(d[6], nd, nrho, tp, no);
     d[7] = relax_plus(d[7], wd, rho, tm, no);
 }
 
 // The collision above in FP32 on one node (V = float) or on two nodes at once
 // (V = float2: lane x one node, lane y the other).  Operation order chosen
-// for accuracy and count (48 operations per node): over 5000 steps of the
-// 4096 x 4 second-sound pulse (Kn_R = 0.1) the max error against FP64 is
-// 6.2e-6 (7.1e-6 with sigma t_i as a separate term, 56 operations; 1.2e-5
-// with w rho also rounded apart from t_i), and 6.6e-8 against 8.1e-7 at
-// 300 steps of the 8192 x 8192 heat mode.  Folding omega into the weights
+// for accuracy and count (48 operations per node, one of them, the negation
+// of rho, held in the negated weights: 424 -> 435 GLUPS on the 8192^2 march
+// of 5 steps): over 5000 steps of the 4096 x 4 second-sound pulse (Kn_R = 0.1)
+// the max error against FP64 is 6.2e-6 (7.1e-6 with sigma t_i as a separate
+// term, 56 operations; 1.2e-5 with w rho also rounded apart from t_i), and
+// 6.6e-8 against 8.1e-7 at 300 steps of the 8192 x 8192 heat mode.  Folding
+// omega into the weights
 // instead (d* = (1 - omega) d + omega eq, 41 operations) loses the small
 // differences d - eq: about 80 times less accurate at Kn_R = 1 and 10 on the
 // second-sound pulse (FP32 emulated on the host).

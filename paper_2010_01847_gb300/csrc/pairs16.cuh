@@ -110,7 +110,7 @@ __device__ __forceinline__ void collide_words16(uint4 (&w)[8], const Coef<float>
         if (m == 1) { r01 = f_add(r01, rho); x01 = f_add(x01, mx); y01 = f_add(y01, my); }
         if (m == 2) { r23 = rho; x23 = mx; y23 = my; }
         if (m == 3) { r23 = f_add(r23, rho); x23 = f_add(x23, mx); y23 = f_add(y23, my); }
-        relax_f32(f, rho, mx, my, k);
+        relax_f32<float2, false>(f, rho, mx, my, k);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
             set_word(w[i], m,
