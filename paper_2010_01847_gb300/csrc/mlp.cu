@@ -21,12 +21,8 @@
 namespace plbm {
 namespace {
 
-constexpr int TK = 32;                     // k depth of a block tile
+constexpr int TK = 64;                     // k depth of a pipeline stage
 constexpr int GEMM_THREADS = 128;          // 4 warps
-
-__device__ __forceinline__ unsigned pack_bf16(__nv_bfloat16 lo, __nv_bfloat16 hi) {
-    return (unsigned)__bfloat16_as_ushort(lo) | ((unsigned)__bfloat16_as_ushort(hi) << 16);
-}
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4],
                                          const unsigned (&b)[2]) {
@@ -48,191 +44,302 @@ __device__ __forceinline__ float gelu_grad(float x) {
 
 enum { EPI_NONE = 0, EPI_GELU = 1, EPI_GELU_BWD = 2 };
 
-// C[m, n] = sum_k A(m, k) B(k, n) (+ bias[n]) with A(m, k) = A[m*am + k*ak],
-// B(k, n) = B[k*bk + n*bn] (any strides: every transposition the forward and
-// backward passes need).  Outputs (each optional): pre = the FP32 result,
-// out = the FP32 result after the epilogue, outb = the same in BF16.
-// Epilogues: GELU (forward), GELU backward (the result times GELU'(aux[m, n]),
-// aux the pre-activation of the layer below: dZ = dX (.) GELU'(Z)).
-// Block tile BM x BN (64 or 32 each), four warps of (BM / 2) x (BN / 2).
-template <int BM, int BN>
-__global__ void __launch_bounds__(GEMM_THREADS)
-gemm_bf16(const __nv_bfloat16 *__restrict__ A, long long am, long long ak,
-          const __nv_bfloat16 *__restrict__ B, long long bk, long long bn,
-          const float *__restrict__ bias, int M, int N, int K, int epi,
-          const float *__restrict__ aux, float *__restrict__ pre, float *__restrict__ out,
-          __nv_bfloat16 *__restrict__ outb) {
-    __shared__ __align__(16) __nv_bfloat16 As[BM][TK + 8];
-    __shared__ __align__(16) __nv_bfloat16 Bs[BN][TK + 8];     // stored [n][k]
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int MI = BM / 32, NJ = BN / 16;     // m16 x n8 tiles per warp
-    const int wm = (warp >> 1) * (BM / 2), wn = (warp & 1) * (BN / 2);
-    const int g = lane >> 2, tg = lane & 3;
-    float acc[MI][NJ][4] = {};
-    const __nv_bfloat16 zero = __float2bfloat16(0.f);
-    // The tiles are filled along the operand's contiguous index with 16-byte
-    // loads (8 values) where the rows are 16-byte aligned, element by element
-    // otherwise (the first layer's 3 inputs) and at the matrix edges.
-    const bool a_k_vec = ak == 1 && am % 8 == 0 && ((uintptr_t)A & 15) == 0;
-    const bool a_m_vec = am == 1 && ak % 8 == 0 && ((uintptr_t)A & 15) == 0;
-    const bool b_k_vec = bk == 1 && bn % 8 == 0 && ((uintptr_t)B & 15) == 0;
-    const bool b_n_vec = bn == 1 && bk % 8 == 0 && ((uintptr_t)B & 15) == 0;
-    for (int k0 = 0; k0 < K; k0 += TK) {
-        if (a_k_vec) {
-            for (int idx = threadIdx.x; idx < BM * TK / 8; idx += GEMM_THREADS) {
-                const int r = idx / (TK / 8), c = (idx % (TK / 8)) * 8;
-                const int m = m0 + r, k = k0 + c;
-                if (m < M && k + 8 <= K) {
-                    *reinterpret_cast<uint4 *>(&As[r][c]) =
-                        *reinterpret_cast<const uint4 *>(A + (long long)m * am + k);
-                } else {
-                    for (int j = 0; j < 8; ++j)
-                        As[r][c + j] = (m < M && k + j < K) ? A[(long long)m * am + k + j] : zero;
-                }
-            }
-        } else if (a_m_vec) {
-            for (int idx = threadIdx.x; idx < BM * TK / 8; idx += GEMM_THREADS) {
-                const int c = idx / (BM / 8), r = (idx % (BM / 8)) * 8;
-                const int m = m0 + r, k = k0 + c;
-                if (k < K && m + 8 <= M) {
-                    const uint4 v = *reinterpret_cast<const uint4 *>(A + m + (long long)k * ak);
-                    const __nv_bfloat16 *h = reinterpret_cast<const __nv_bfloat16 *>(&v);
-                    for (int j = 0; j < 8; ++j) As[r + j][c] = h[j];
-                } else {
-                    for (int j = 0; j < 8; ++j)
-                        As[r + j][c] = (k < K && m + j < M) ? A[m + j + (long long)k * ak] : zero;
-                }
-            }
-        } else {
-            for (int idx = threadIdx.x; idx < BM * TK; idx += GEMM_THREADS) {
-                const int r = idx / TK, c = idx % TK;
-                const int m = m0 + r, k = k0 + c;
-                As[r][c] = (m < M && k < K) ? A[(long long)m * am + (long long)k * ak] : zero;
-            }
-        }
-        if (b_k_vec) {
-            for (int idx = threadIdx.x; idx < BN * TK / 8; idx += GEMM_THREADS) {
-                const int r = idx / (TK / 8), c = (idx % (TK / 8)) * 8;
-                const int n = n0 + r, k = k0 + c;
-                if (n < N && k + 8 <= K) {
-                    *reinterpret_cast<uint4 *>(&Bs[r][c]) =
-                        *reinterpret_cast<const uint4 *>(B + k + (long long)n * bn);
-                } else {
-                    for (int j = 0; j < 8; ++j)
-                        Bs[r][c + j] = (n < N && k + j < K) ? B[k + j + (long long)n * bn] : zero;
-                }
-            }
-        } else if (b_n_vec) {
-            for (int idx = threadIdx.x; idx < BN * TK / 8; idx += GEMM_THREADS) {
-                const int c = idx / (BN / 8), r = (idx % (BN / 8)) * 8;
-                const int n = n0 + r, k = k0 + c;
-                if (k < K && n + 8 <= N) {
-                    const uint4 v = *reinterpret_cast<const uint4 *>(B + (long long)k * bk + n);
-                    const __nv_bfloat16 *h = reinterpret_cast<const __nv_bfloat16 *>(&v);
-                    for (int j = 0; j < 8; ++j) Bs[r + j][c] = h[j];
-                } else {
-                    for (int j = 0; j < 8; ++j)
-                        Bs[r + j][c] = (k < K && n + j < N) ? B[(long long)k * bk + n + j] : zero;
-                }
-            }
-        } else {
-            for (int idx = threadIdx.x; idx < BN * TK; idx += GEMM_THREADS) {
-                const int r = idx / TK, c = idx % TK;
-                const int n = n0 + r, k = k0 + c;
-                Bs[r][c] = (n < N && k < K) ? B[(long long)k * bk + (long long)n * bn] : zero;
-            }
-        }
-        __syncthreads();
+// Every BF16 matrix has rows of ld = width rounded up to 8 elements (16-byte
+// aligned rows, zeros behind the width), so every tile is filled by 16-byte
+// asynchronous copies whatever the widths.
+__host__ __device__ constexpr long long ld8(long long n) { return (n + 7) & ~7LL; }
+
+// C[m, n] = sum_k A(m, k) B(k, n) (+ bias[n]), FP32, [M x N].  Outputs (each
+// optional): pre = the result, out = the result after the epilogue, outb = the
+// same in BF16 (rows of ld8(N), zeros behind N).  Epilogues: GELU (forward),
+// GELU backward (the result times GELU'(aux[m, n]), aux the pre-activation of
+// the layer below: dZ = dX (.) GELU'(Z)).
+struct Product {
+    const __nv_bfloat16 *A, *B;
+    long long lda, ldb;
+    const float *bias, *aux;
+    float *pre, *out;
+    __nv_bfloat16 *outb;
+    int M, N, K, epi;
+};
+
+// Tile shape of a block's product: T x T outputs, four warps of T/2 x T/2.
+// What bounds these products is latency, not rate: a few hundred rows and
+// columns are one wave of small blocks, and each block's chain is load, wait,
+// multiply.  So a stage is 64 deep and STAGES of them are in flight at once:
+// with T = 32 the whole depth of 512 is requested before the first multiply.
+// With one launch per layer and direction, a training step of the
+// 3-256-256-256-256-512 network at 512 rows takes 72 us; a 32-deep loop that
+// loaded, waited and multiplied in turn, in 24 launches, took 207.
+// A row of a tile is padded by 8 elements (an odd number of 16-byte units:
+// ldmatrix reads 8 rows without bank conflicts).
+template <int T> struct Tile {
+    static constexpr int STAGES = T == 32 ? 8 : 4;
+    static constexpr int K_ROW = TK + 8, M_ROW = T + 8;       // row lengths of the two layouts
+    static constexpr int OPERAND = T * K_ROW > TK * M_ROW ? T * K_ROW : TK * M_ROW;   // elements
+    static constexpr int SMEM = STAGES * 2 * OPERAND * 2;     // bytes
+};
+
+__device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool valid) {
+    const int n = valid ? 16 : 0;                              // 0: zeros
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n)
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm4(unsigned (&r)[4], unsigned addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void ldsm4_t(unsigned (&r)[4], unsigned addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+
+// Copies of one operand's tile for depth k0 .. k0 + TK - 1.  KMAJOR: the
+// operand is stored [line][k] (rows of `lines`, ld >= its depth); else
+// [k][line].  r0: the tile's first line.
+template <int T, bool KMAJOR>
+__device__ __forceinline__ void stage_operand(unsigned dst, const __nv_bfloat16 *src, long long ld,
+                                              int lines, int depth, int r0, int k0) {
 #pragma unroll
-        for (int kk = 0; kk < TK; kk += 16) {
-            unsigned a[MI][4], b[NJ][2];
+    for (int it = 0; it < T * TK / 8 / GEMM_THREADS; ++it) {
+        const int idx = it * GEMM_THREADS + threadIdx.x;
+        if (KMAJOR) {
+            const int r = idx / (TK / 8), c = (idx % (TK / 8)) * 8;
+            const bool ok = r0 + r < lines && k0 + c < depth;   // a chunk past depth: zeros
+            const long long o = ok ? (long long)(r0 + r) * ld + k0 + c : 0;
+            cp_async16(dst + 2 * (r * Tile<T>::K_ROW + c), src + o, ok);
+        } else {
+            const int k = idx / (T / 8), c = (idx % (T / 8)) * 8;
+            const bool ok = k0 + k < depth && r0 + c < lines;
+            const long long o = ok ? (long long)(k0 + k) * ld + r0 + c : 0;
+            cp_async16(dst + 2 * (k * Tile<T>::M_ROW + c), src + o, ok);
+        }
+    }
+}
+
+// The T x T tile at (m0, n0) of one product; every thread of the block calls
+// it.  The depth is summed in k order, 16 at a time, whatever the tile.
+template <int T, bool A_KMAJOR, bool B_KMAJOR>
+__device__ __forceinline__ void product_tile(const Product &g, int m0, int n0, unsigned smem) {
+    constexpr int MI = T / 32, NJ = T / 16;       // m16 and n8 tiles per warp
+    constexpr int STAGES = Tile<T>::STAGES;
+    constexpr unsigned OP = Tile<T>::OPERAND * 2;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int wm = (warp >> 1) * (T / 2), wn = (warp & 1) * (T / 2);
+    const int gr = lane >> 2, tg = lane & 3;
+    const int chunks = (g.K + TK - 1) / TK;
+    auto stage = [&](int c) {
+        if (c < chunks) {
+            const unsigned a = smem + (c % STAGES) * 2 * OP;
+            stage_operand<T, A_KMAJOR>(a, g.A, g.lda, g.M, g.K, m0, c * TK);
+            stage_operand<T, B_KMAJOR>(a + OP, g.B, g.ldb, g.N, g.K, n0, c * TK);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int c = 0; c < STAGES - 1; ++c) stage(c);
+    // the lane's row address in each operand's tile (see ldmatrix)
+    const int j = lane >> 3, r = lane & 7;
+    const unsigned a_at = A_KMAJOR ? 2 * ((wm + (lane & 15)) * Tile<T>::K_ROW + (lane >> 4) * 8)
+                                   : 2 * (((j >> 1) * 8 + r) * Tile<T>::M_ROW + wm + (j & 1) * 8);
+    const unsigned b_at = B_KMAJOR ? 2 * ((wn + (j >> 1) * 8 + r) * Tile<T>::K_ROW + (j & 1) * 8)
+                                   : 2 * (((j & 1) * 8 + r) * Tile<T>::M_ROW + wn + (j >> 1) * 8);
+    constexpr unsigned A_I = 2 * 16 * (A_KMAJOR ? Tile<T>::K_ROW : 1);     // next 16 lines
+    constexpr unsigned B_J = 2 * 16 * (B_KMAJOR ? Tile<T>::K_ROW : 1);
+    constexpr unsigned A_K = 2 * 16 * (A_KMAJOR ? 1 : Tile<T>::M_ROW);     // next 16 of the depth
+    constexpr unsigned B_K = 2 * 16 * (B_KMAJOR ? 1 : Tile<T>::M_ROW);
+    float acc[MI][NJ][4] = {};
+    for (int c = 0; c < chunks; ++c) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+        __syncthreads();              // stage c is there, stage c - 1 is read by all
+        stage(c + STAGES - 1);
+        const unsigned sa = smem + (c % STAGES) * 2 * OP, sb = sa + OP;
+#pragma unroll
+        for (int kk = 0; kk < TK / 16; ++kk) {
+            if (c * TK + kk * 16 >= g.K) break;
+            unsigned a[MI][4], b[NJ / 2][4];
 #pragma unroll
             for (int i = 0; i < MI; ++i) {
-                const int r = wm + 16 * i + g;
-                a[i][0] = pack_bf16(As[r][kk + 2 * tg], As[r][kk + 2 * tg + 1]);
-                a[i][1] = pack_bf16(As[r + 8][kk + 2 * tg], As[r + 8][kk + 2 * tg + 1]);
-                a[i][2] = pack_bf16(As[r][kk + 2 * tg + 8], As[r][kk + 2 * tg + 9]);
-                a[i][3] = pack_bf16(As[r + 8][kk + 2 * tg + 8], As[r + 8][kk + 2 * tg + 9]);
+                const unsigned at = sa + a_at + i * A_I + kk * A_K;
+                if (A_KMAJOR) ldsm4(a[i], at);
+                else ldsm4_t(a[i], at);
             }
 #pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                const int c = wn + 8 * j + g;
-                b[j][0] = pack_bf16(Bs[c][kk + 2 * tg], Bs[c][kk + 2 * tg + 1]);
-                b[j][1] = pack_bf16(Bs[c][kk + 2 * tg + 8], Bs[c][kk + 2 * tg + 9]);
+            for (int q = 0; q < NJ / 2; ++q) {
+                const unsigned at = sb + b_at + q * B_J + kk * B_K;
+                if (B_KMAJOR) ldsm4(b[q], at);
+                else ldsm4_t(b[q], at);
             }
 #pragma unroll
             for (int i = 0; i < MI; ++i)
 #pragma unroll
-                for (int j = 0; j < NJ; ++j) mma_bf16(acc[i][j], a[i], b[j]);
+                for (int q = 0; q < NJ; ++q) {
+                    const unsigned bq[2] = {b[q / 2][(q & 1) * 2], b[q / 2][(q & 1) * 2 + 1]};
+                    mma_bf16(acc[i][q], a[i], bq);
+                }
         }
-        __syncthreads();
     }
+    const long long ldo = ld8(g.N);
 #pragma unroll
     for (int i = 0; i < MI; ++i)
 #pragma unroll
-        for (int j = 0; j < NJ; ++j)
+        for (int q = 0; q < NJ; ++q)
 #pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                const int m = m0 + wm + 16 * i + g + (h >= 2 ? 8 : 0);
-                const int n = n0 + wn + 8 * j + 2 * tg + (h & 1);
-                if (m >= M || n >= N) continue;
-                float v = acc[i][j][h] + (bias ? bias[n] : 0.f);
-                const long long o = (long long)m * N + n;
-                if (pre) pre[o] = v;
-                if (epi == EPI_GELU) v = gelu(v);
-                if (epi == EPI_GELU_BWD) v = v * gelu_grad(aux[o]);
-                if (out) out[o] = v;
-                if (outb) outb[o] = __float2bfloat16_rn(v);
+            for (int h = 0; h < 2; ++h) {         // rows g, g + 8: two adjacent columns each
+                const int m = m0 + wm + 16 * i + gr + 8 * h;
+                const int n = n0 + wn + 8 * q + 2 * tg;
+                if (m >= g.M || n >= ldo) continue;
+                float v[2] = {0.f, 0.f};
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    if (n + e >= g.N) continue;
+                    const long long o = (long long)m * g.N + n + e;
+                    v[e] = acc[i][q][2 * h + e] + (g.bias ? g.bias[n + e] : 0.f);
+                    if (g.pre) g.pre[o] = v[e];
+                    if (g.epi == EPI_GELU) v[e] = gelu(v[e]);
+                    if (g.epi == EPI_GELU_BWD) v[e] = v[e] * gelu_grad(g.aux[o]);
+                    if (g.out) g.out[o] = v[e];
+                }
+                if (g.outb)
+                    *reinterpret_cast<__nv_bfloat162 *>(g.outb + (long long)m * ldo + n) =
+                        __floats2bfloat162_rn(v[0], v[1]);
             }
 }
 
-__global__ void to_bf16(const float *__restrict__ x, __nv_bfloat16 *__restrict__ y, long long n) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        y[i] = __float2bfloat16_rn(x[i]);
+__host__ __device__ constexpr long long tiles_of(long long n, int t) { return (n + t - 1) / t; }
+
+// Forward product of a layer: A = X [M x K], B(k, n) = W[n][k].
+template <int T>
+__global__ void __launch_bounds__(GEMM_THREADS) forward_product(const Product g) {
+    extern __shared__ __align__(16) unsigned char tiles[];
+    const int tn = (int)tiles_of(g.N, T);
+    const int bm = blockIdx.x / tn, bn = blockIdx.x - bm * tn;
+    product_tile<T, true, true>(g, bm * T, bn * T, (unsigned)__cvta_generic_to_shared(tiles));
 }
 
-// dY = 2 (Y - T) / (B N) (mean squared error), and the loss partial sums.
-__global__ void mse_grad(const float *__restrict__ y, const float *__restrict__ t, long long n,
-                         float scale, float *__restrict__ dy, __nv_bfloat16 *__restrict__ dyb,
-                         double *__restrict__ loss_partials) {
+// db[n] = sum over the batch of dZ[b, n]: 8 rows' worth of partial sums, sum
+// w over rows w, w + 8, ... in order, then the 8 sums in order: a fixed order,
+// so the result does not vary between runs.  A block takes 16 columns (thread
+// w * 16 + column); its loads do not depend on the running sums, 32 in flight.
+constexpr int BIAS_SUMS = 8, BIAS_COLS = GEMM_THREADS / BIAS_SUMS;
+__device__ __forceinline__ void bias_block(const float *__restrict__ dz, int B, int N, int n0,
+                                           float *__restrict__ db, float *part) {
+    const int col = threadIdx.x % BIAS_COLS, w = threadIdx.x / BIAS_COLS, n = n0 + col;
+    float s = 0.f;
+    if (n < N) {
+#pragma unroll 32
+        for (int b = w; b < B; b += BIAS_SUMS) s += dz[(long long)b * N + n];
+    }
+    part[threadIdx.x] = s;
+    __syncthreads();
+    if (w == 0 && n < N) {
+        float t = 0.f;
+#pragma unroll
+        for (int i = 0; i < BIAS_SUMS; ++i) t += part[i * BIAS_COLS + col];
+        db[n] = t;
+    }
+}
+
+// Everything of a layer's backward pass that needs its dZ, in one launch:
+// blocks [0, nw): dW = dZ^T X (w); [nw, nw + nx): dZ of the layer below (x,
+// dX (.) GELU'); the rest: the bias gradient.  One launch in place of three
+// in turn: each is a fraction of a wave (64, 128 and 16 blocks for the hidden
+// layers at 512 rows).
+template <int T>
+__global__ void __launch_bounds__(GEMM_THREADS)
+backward_products(const Product w, const Product x, long long nw, long long nx,
+                  const float *__restrict__ dz, int batch, int N, float *__restrict__ db) {
+    extern __shared__ __align__(16) unsigned char tiles[];
+    const unsigned smem = (unsigned)__cvta_generic_to_shared(tiles);
+    const long long id = blockIdx.x;
+    if (id < nw) {
+        const int tn = (int)tiles_of(w.N, T);
+        const int bm = int(id / tn), bn = int(id - (long long)bm * tn);
+        product_tile<T, false, false>(w, bm * T, bn * T, smem);
+    } else if (id < nw + nx) {
+        const int tn = (int)tiles_of(x.N, T);
+        const int bm = int((id - nw) / tn), bn = int((id - nw) - (long long)bm * tn);
+        product_tile<T, true, false>(x, bm * T, bn * T, smem);
+    } else {
+        bias_block(dz, batch, N, int(id - nw - nx) * BIAS_COLS, db, (float *)tiles);
+    }
+}
+
+// Rows of n FP32 values as rows of ld8(n) BF16 values.
+__global__ void to_bf16_rows(const float *__restrict__ x, __nv_bfloat16 *__restrict__ y,
+                             long long rows, int n) {
+    const long long ld = ld8(n), total = rows * ld;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += (long long)gridDim.x * blockDim.x) {
+        const long long r = i / ld;
+        const int c = int(i - r * ld);
+        y[i] = __float2bfloat16_rn(c < n ? x[r * n + c] : 0.f);
+    }
+}
+
+// SplitMix64 (Steele, Lea and Flood's generator) of a 64-bit counter.
+__device__ __forceinline__ unsigned long long splitmix64(unsigned long long z) {
+    z += 0x9E3779B97F4A7C15ULL;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
+    return z ^ (z >> 31);
+}
+
+// Per-step scalars of the device training loop (train_setup writes them).
+struct TrainState {
+    long long t;          // Adam steps taken so far (all calls)
+    long long local;      // steps of this call so far: the step being run, until train_setup
+    float lr, c1, c2;     // learning rate and bias corrections of the step
+};
+
+// The minibatch of a training step: row j is sample (batch >= n ? j :
+// SplitMix64(seed ^ (step batch + j)) mod n), drawn with replacement.
+// st == nullptr: row j is sample j.
+struct Minibatch {
+    const TrainState *st;
+    unsigned long long seed;
+    int n, batch;
+};
+__device__ __forceinline__ long long sample_of(const Minibatch &mb, long long base, int j) {
+    if (!mb.st || mb.batch >= mb.n) return j;
+    return (long long)(splitmix64(mb.seed ^ ((unsigned long long)base + (unsigned)j)) %
+                       (unsigned long long)mb.n);
+}
+
+// The step's input rows, in BF16.
+__global__ void gather_rows(const float *__restrict__ x, int kx, Minibatch mb,
+                            __nv_bfloat16 *__restrict__ y) {
+    const long long ld = ld8(kx), total = mb.batch * ld, base = mb.st->local * mb.batch;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += (long long)gridDim.x * blockDim.x) {
+        const int j = int(i / ld), c = int(i - j * ld);
+        y[i] = __float2bfloat16_rn(c < kx ? x[sample_of(mb, base, j) * kx + c] : 0.f);
+    }
+}
+
+// dY = 2 (Y - T) / (B N) (mean squared error), FP32 [B x N] and BF16 (rows of
+// ld8(N)), and the loss partial sums.
+__global__ void mse_grad(const float *__restrict__ y, const float *__restrict__ t, int rows, int N,
+                         Minibatch mb, float scale, float *__restrict__ dy,
+                         __nv_bfloat16 *__restrict__ dyb, double *__restrict__ loss_partials) {
+    const long long n = (long long)rows * N, base = mb.st ? mb.st->local * mb.batch : 0;
+    const int ld = (int)ld8(N);
     double s = 0.0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
-        const float d = y[i] - t[i];
+        const int j = int(i / N), c = int(i - (long long)j * N);
+        const float d = y[i] - t[sample_of(mb, base, j) * N + c];
         s += (double)(d * d);
         const float gval = 2.0f * d * scale;
         dy[i] = gval;
-        dyb[i] = __float2bfloat16_rn(gval);
+        dyb[(long long)j * ld + c] = __float2bfloat16_rn(gval);
+        if (c == N - 1)
+            for (int z = N; z < ld; ++z) dyb[(long long)j * ld + z] = __float2bfloat16_rn(0.f);
     }
     double acc[5] = {s, 0.0, 0.0, 0.0, 0.0};
     block_sum5_store(acc, loss_partials + (size_t)blockIdx.x * 5);
-}
-
-// db[n] = sum over the batch of dZ[b, n]: a block of 8 warps per 32
-// columns, warp w summing rows w, w + 8, ... (lanes on consecutive columns,
-// loads independent of the running sums), then the 8 warp sums added in
-// warp order: a fixed order, so the result does not vary between runs.
-constexpr int BIAS_WARPS = 8;
-__global__ void __launch_bounds__(32 * BIAS_WARPS)
-bias_grad(const float *__restrict__ dz, int B, int N, float *__restrict__ db) {
-    __shared__ float part[BIAS_WARPS][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int n = blockIdx.x * 32 + lane;
-    float s = 0.f;
-    if (n < N) {
-#pragma unroll 8
-        for (int b = warp; b < B; b += BIAS_WARPS) s += dz[(long long)b * N + n];
-    }
-    part[warp][lane] = s;
-    __syncthreads();
-    if (warp == 0 && n < N) {
-        float t = 0.f;
-#pragma unroll
-        for (int w = 0; w < BIAS_WARPS; ++w) t += part[w][lane];
-        db[n] = t;
-    }
 }
 
 // One Adam update of parameter i (refreshing its BF16 copy if it is a weight).
@@ -262,20 +369,14 @@ __global__ void adam(float *__restrict__ p, const float *__restrict__ g, float *
         adam_update(i, p, g, m, v, lr, b1, b2, eps, c1, c2, wmap, pb);
 }
 
-// Per-step scalars of the device training loop (train_setup writes them).
-struct TrainState {
-    long long t;          // Adam steps taken so far (all calls)
-    long long local;      // steps of this call so far
-    long long cur;        // the step being run (this call's numbering)
-    float lr, c1, c2;     // learning rate and bias corrections of the step
-};
-
-// One thread: the step's learning rate (cosine from lr to lr_final over
-// `steps`) and Adam's bias corrections 1 - beta^t, then the counters.
+// One thread: the step's loss (mean of the squared errors) into the history,
+// its learning rate (cosine from lr to lr_final over `steps`) and Adam's bias
+// corrections 1 - beta^t, then the counters.
 __global__ void train_setup(TrainState *st, long long steps, float lr, float lr_final,
-                            float b1, float b2) {
+                            float b1, float b2, const double *__restrict__ total, double inv_n,
+                            float *__restrict__ hist) {
     const long long t = st->t + 1, s = st->local;
-    st->cur = s;
+    hist[s] = (float)(*total * inv_n);
     st->lr = (float)((double)lr_final +
                      0.5 * ((double)lr - (double)lr_final) *
                          (1.0 + cos(3.14159265358979323846 * (double)s / (double)steps)));
@@ -283,41 +384,6 @@ __global__ void train_setup(TrainState *st, long long steps, float lr, float lr_
     st->c2 = 1.f - (float)pow((double)b2, (double)t);
     st->t = t;
     st->local = s + 1;
-}
-
-// SplitMix64 (Steele, Lea and Flood's generator) of a 64-bit counter.
-__device__ __forceinline__ unsigned long long splitmix64(unsigned long long z) {
-    z += 0x9E3779B97F4A7C15ULL;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
-    return z ^ (z >> 31);
-}
-
-// The step's minibatch: row j is sample (batch >= n ? j : SplitMix64(seed ^
-// (step batch + j)) mod n), drawn with replacement; rows of x [n x kx] and
-// t [n x kt] are copied to xb and tb.
-__global__ void gather_rows(const float *__restrict__ x, const float *__restrict__ t, int n,
-                            int kx, int kt, int batch, unsigned long long seed,
-                            const TrainState *__restrict__ st, float *__restrict__ xb,
-                            float *__restrict__ tb) {
-    const int kw = kx > kt ? kx : kt;
-    const long long total = (long long)batch * kw;
-    const unsigned long long base = (unsigned long long)st->cur * (unsigned long long)batch;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(i / kw), c = (int)(i - (long long)j * kw);
-        const long long src = batch >= n ? j
-                                         : (long long)(splitmix64(seed ^ (base + (unsigned)j)) %
-                                                       (unsigned long long)n);
-        if (c < kx) xb[(long long)j * kx + c] = x[src * kx + c];
-        if (c < kt) tb[(long long)j * kt + c] = t[src * kt + c];
-    }
-}
-
-// The step's loss (mean of the squared errors) into the history.
-__global__ void record_loss(const double *__restrict__ total, double inv_n,
-                            const TrainState *__restrict__ st, float *__restrict__ hist) {
-    hist[st->cur] = (float)(*total * inv_n);
 }
 
 // Adam with the step's scalars from the device (the training loop).
@@ -353,15 +419,16 @@ struct lbm_mlp {
     float *params = nullptr, *grads = nullptr, *m = nullptr, *v = nullptr;
     __nv_bfloat16 *wb = nullptr;          // BF16 weights
     long long *wmap = nullptr;            // flat index -> BF16 index (or -1)
-    std::vector<float *> pre;             // pre-activations per layer [B x N_l]
-    std::vector<float *> act;             // FP32 outputs per layer
+    std::vector<float *> pre;             // pre-activations per hidden layer [B x N_l]
+    float *act = nullptr;                 // FP32 output of the last layer
     std::vector<__nv_bfloat16 *> actb;    // BF16 layer inputs: actb[0] = X, actb[l+1] = out of l
     float *g0 = nullptr, *g1 = nullptr;   // gradient ping-pong [B x max width]
     __nv_bfloat16 *gb = nullptr, *gb1 = nullptr;   // BF16 copies of the two
-    // device training loop: state, gathered minibatch, capture stream
+    // device training loop: state, capture streams (the second takes the
+    // step's loss and scalars beside the backward pass) and their events
     TrainState *tstate = nullptr;
-    float *xb = nullptr, *tb = nullptr;
-    cudaStream_t cap = nullptr;
+    cudaStream_t cap = nullptr, cap2 = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
     double *loss_part = nullptr;
     long long steps = 0;
     std::string err;
@@ -387,68 +454,125 @@ lbm_status mcuda(lbm_mlp *m, cudaError_t e, const char *where) {
         if (e_ != cudaSuccess) return mcuda(m, e_, #call);     \
     } while (0)
 
-cudaError_t gemm(cudaStream_t s, const __nv_bfloat16 *A, long long am, long long ak,
-                 const __nv_bfloat16 *B, long long bk, long long bn, const float *bias, int M,
-                 int N, int K, int epi, const float *aux, float *pre, float *out,
-                 __nv_bfloat16 *outb) {
-    // 64 x 64 tiles when they give at least two blocks per SM, else 32 x 32
-    // (the network's products are small: a few hundred rows and columns)
-    const long long big = (long long)((N + 63) / 64) * ((M + 63) / 64);
-    if (big >= 2 * 152) {
-        dim3 grid((N + 63) / 64, (M + 63) / 64);
-        gemm_bf16<64, 64><<<grid, GEMM_THREADS, 0, s>>>(A, am, ak, B, bk, bn, bias, M, N, K,
-                                                        epi, aux, pre, out, outb);
-    } else {
-        dim3 grid((N + 31) / 32, (M + 31) / 32);
-        gemm_bf16<32, 32><<<grid, GEMM_THREADS, 0, s>>>(A, am, ak, B, bk, bn, bias, M, N, K,
-                                                        epi, aux, pre, out, outb);
-    }
+// 64 x 64 tiles when they give at least two blocks per SM, else 32 x 32 (the
+// network's products are small: a few hundred rows and columns).
+constexpr long long BIG_TILES = 2 * 152;
+
+template <int T> cudaError_t launch_forward(const Product &g, cudaStream_t s) {
+    const long long blocks = tiles_of(g.M, T) * tiles_of(g.N, T);
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    cudaError_t e = cudaFuncSetAttribute(forward_product<T>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         Tile<T>::SMEM);
+    if (e != cudaSuccess) return e;
+    forward_product<T><<<(unsigned)blocks, GEMM_THREADS, Tile<T>::SMEM, s>>>(g);
     return cudaGetLastError();
 }
 
-// Forward pass of `batch` rows of X (FP32 device [batch x K_0]) on stream
-// s; the output layer's FP32 result is act[L-1].
-cudaError_t forward(lbm_mlp *m, const float *x, int batch, cudaStream_t s) {
-    to_bf16<<<grid1((long long)batch * m->widths[0]), 256, 0, s>>>(
-        x, m->actb[0], (long long)batch * m->widths[0]);
-    cudaError_t e = cudaGetLastError();
+template <int T>
+cudaError_t launch_backward(const Product &w, const Product &x, const float *dz, int batch, int N,
+                            float *db, cudaStream_t s) {
+    const long long nw = tiles_of(w.M, T) * tiles_of(w.N, T);
+    const long long nx = x.A ? tiles_of(x.M, T) * tiles_of(x.N, T) : 0;
+    const long long blocks = nw + nx + tiles_of(N, BIAS_COLS);
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    cudaError_t e = cudaFuncSetAttribute(backward_products<T>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         Tile<T>::SMEM);
+    if (e != cudaSuccess) return e;
+    backward_products<T><<<(unsigned)blocks, GEMM_THREADS, Tile<T>::SMEM, s>>>(w, x, nw, nx, dz,
+                                                                               batch, N, db);
+    return cudaGetLastError();
+}
+
+// The layers on the `batch` BF16 rows in actb[0], on stream s; the output
+// layer's FP32 result is act[L-1].
+cudaError_t forward_layers(lbm_mlp *m, int batch, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
     for (int l = 0; l < m->layers && e == cudaSuccess; ++l) {
         const int K = m->widths[l], N = m->widths[l + 1];
         const bool last = l == m->layers - 1;
-        e = gemm(s, m->actb[l], K, 1, m->wb + m->wb_off[l], 1, K, m->params + m->b_off[l], batch,
-                 N, K, last ? EPI_NONE : EPI_GELU, nullptr, m->pre[l], m->act[l],
-                 last ? nullptr : m->actb[l + 1]);
+        Product g{};
+        g.A = m->actb[l];
+        g.lda = ld8(K);
+        g.B = m->wb + m->wb_off[l];
+        g.ldb = ld8(K);
+        g.bias = m->params + m->b_off[l];
+        g.pre = last ? nullptr : m->pre[l];
+        g.out = last ? m->act : nullptr;
+        g.outb = last ? nullptr : m->actb[l + 1];
+        g.M = batch;
+        g.N = N;
+        g.K = K;
+        g.epi = last ? EPI_NONE : EPI_GELU;
+        e = tiles_of(batch, 64) * tiles_of(N, 64) >= BIG_TILES ? launch_forward<64>(g, s)
+                                                               : launch_forward<32>(g, s);
     }
     return e;
 }
 
-// Loss partial sums and every parameter's gradient (into m->grads) for
-// targets t of the rows forward() last ran, on stream s; no host copy, no
-// synchronisation.  The total loss (sum of squares) lands at
-// loss_part[5 * 4096].
-cudaError_t backward(lbm_mlp *m, const float *t, int batch, cudaStream_t s) {
-    const int L = m->layers;
-    const long long no = (long long)batch * m->widths[L];
-    const unsigned gl = grid1(no);
-    mse_grad<<<gl, 256, 0, s>>>(m->act[L - 1], t, no, 1.0f / (float)no, m->g0, m->gb,
-                                m->loss_part);
+// Forward pass of `batch` rows of X (FP32 device [batch x K_0]) on stream s.
+cudaError_t forward(lbm_mlp *m, const float *x, int batch, cudaStream_t s) {
+    to_bf16_rows<<<grid1((long long)batch * m->widths[0]), 256, 0, s>>>(x, m->actb[0], batch,
+                                                                        m->widths[0]);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = launch_finalize(m->loss_part, (int)gl, m->loss_part + 5 * 4096, s);
+    return e == cudaSuccess ? forward_layers(m, batch, s) : e;
+}
+
+// dY of the rows the forward pass last ran against targets t (of mb's
+// samples), and the loss partial sums.
+cudaError_t output_grad(lbm_mlp *m, const float *t, int batch, const Minibatch &mb,
+                        cudaStream_t s) {
+    const int N = m->widths[m->layers];
+    const long long no = (long long)batch * N;
+    mse_grad<<<grid1(no), 256, 0, s>>>(m->act, t, batch, N, mb, 1.0f / (float)no, m->g0, m->gb,
+                                       m->loss_part);
+    return cudaGetLastError();
+}
+
+// The total loss (sum of squares) into loss_part[5 * 4096].
+cudaError_t total_loss(lbm_mlp *m, int batch, cudaStream_t s) {
+    return launch_finalize(m->loss_part, (int)grid1((long long)batch * m->widths[m->layers]),
+                           m->loss_part + 5 * 4096, s);
+}
+
+// Every parameter's gradient (into m->grads) after output_grad, on stream s;
+// no host copy, no synchronisation.
+cudaError_t backward(lbm_mlp *m, int batch, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
     float *g = m->g0, *gn = m->g1;
     __nv_bfloat16 *gbf = m->gb, *gbn = m->gb1;
-    for (int l = L - 1; l >= 0 && e == cudaSuccess; --l) {
+    for (int l = m->layers - 1; l >= 0 && e == cudaSuccess; --l) {
         const int K = m->widths[l], N = m->widths[l + 1];
         // dW_l = dZ_l^T X_l   ([N x K], sum over the batch)
-        e = gemm(s, gbf, 1, N, m->actb[l], K, 1, nullptr, N, K, batch, EPI_NONE, nullptr,
-                 nullptr, m->grads + m->w_off[l], nullptr);
-        if (e != cudaSuccess) break;
-        bias_grad<<<(N + 31) / 32, 32 * BIAS_WARPS, 0, s>>>(g, batch, N, m->grads + m->b_off[l]);
-        e = cudaGetLastError();
-        if (l == 0 || e != cudaSuccess) break;
-        // dZ_{l-1} = (dZ_l W_l) (.) GELU'(Z_{l-1})   ([B x K], the GELU of
-        // layer l - 1 in the product's epilogue)
-        e = gemm(s, gbf, N, 1, m->wb + m->wb_off[l], K, 1, nullptr, batch, K, N, EPI_GELU_BWD,
-                 m->pre[l - 1], nullptr, gn, gbn);
+        Product w{}, x{};
+        w.A = gbf;
+        w.lda = ld8(N);
+        w.B = m->actb[l];
+        w.ldb = ld8(K);
+        w.out = m->grads + m->w_off[l];
+        w.M = N;
+        w.N = K;
+        w.K = batch;
+        long long big = tiles_of(N, 64) * tiles_of(K, 64);
+        if (l > 0) {
+            // dZ_{l-1} = (dZ_l W_l) (.) GELU'(Z_{l-1})   ([B x K], the GELU of
+            // layer l - 1 in the product's epilogue)
+            x.A = gbf;
+            x.lda = ld8(N);
+            x.B = m->wb + m->wb_off[l];
+            x.ldb = ld8(K);
+            x.aux = m->pre[l - 1];
+            x.out = gn;
+            x.outb = gbn;
+            x.M = batch;
+            x.N = K;
+            x.K = N;
+            x.epi = EPI_GELU_BWD;
+            big += tiles_of(batch, 64) * tiles_of(K, 64);
+        }
+        e = big >= BIG_TILES ? launch_backward<64>(w, x, g, batch, N, m->grads + m->b_off[l], s)
+                             : launch_backward<32>(w, x, g, batch, N, m->grads + m->b_off[l], s);
         std::swap(g, gn);
         std::swap(gbf, gbn);
     }
@@ -482,7 +606,7 @@ lbm_status lbm_mlp_create(const int *widths, int n_widths, int max_batch, void *
         m->b_off.push_back(m->n_params);
         m->n_params += N;
         m->wb_off.push_back(m->n_wb);
-        m->n_wb += (long long)N * K;
+        m->n_wb += (long long)N * ld8(K);
     }
     for (int i = 0; i < n_widths; ++i) wmax = std::max(wmax, widths[i]);
     cudaError_t e = cudaSuccess;
@@ -496,24 +620,23 @@ lbm_status lbm_mlp_create(const int *widths, int n_widths, int max_batch, void *
     al((void **)&m->wb, sizeof(__nv_bfloat16) * m->n_wb);
     al((void **)&m->wmap, sizeof(long long) * m->n_params);
     m->pre.assign(m->layers, nullptr);
-    m->act.assign(m->layers, nullptr);
-    m->actb.assign(m->layers + 1, nullptr);
+    m->actb.assign(m->layers, nullptr);
     for (int l = 0; l < m->layers; ++l) {
-        al((void **)&m->pre[l], sizeof(float) * (size_t)max_batch * widths[l + 1]);
-        al((void **)&m->act[l], sizeof(float) * (size_t)max_batch * widths[l + 1]);
+        float **o = l < m->layers - 1 ? &m->pre[l] : &m->act;
+        al((void **)o, sizeof(float) * (size_t)max_batch * widths[l + 1]);
+        al((void **)&m->actb[l], sizeof(__nv_bfloat16) * (size_t)max_batch * ld8(widths[l]));
     }
-    for (int l = 0; l <= m->layers; ++l)
-        al((void **)&m->actb[l], sizeof(__nv_bfloat16) * (size_t)max_batch * widths[l]);
     al((void **)&m->g0, sizeof(float) * (size_t)max_batch * wmax);
     al((void **)&m->g1, sizeof(float) * (size_t)max_batch * wmax);
-    al((void **)&m->gb, sizeof(__nv_bfloat16) * (size_t)max_batch * wmax);
-    al((void **)&m->gb1, sizeof(__nv_bfloat16) * (size_t)max_batch * wmax);
+    al((void **)&m->gb, sizeof(__nv_bfloat16) * (size_t)max_batch * ld8(wmax));
+    al((void **)&m->gb1, sizeof(__nv_bfloat16) * (size_t)max_batch * ld8(wmax));
     al((void **)&m->loss_part, sizeof(double) * 5 * 4097);   // partials + total
     if (e == cudaSuccess) {
         std::vector<long long> map(m->n_params, -1);
         for (int l = 0; l < m->layers; ++l) {
-            const long long nw = (long long)widths[l] * widths[l + 1];
-            for (long long i = 0; i < nw; ++i) map[m->w_off[l] + i] = m->wb_off[l] + i;
+            const long long K = widths[l], nw = K * widths[l + 1];
+            for (long long i = 0; i < nw; ++i)
+                map[m->w_off[l] + i] = m->wb_off[l] + i / K * ld8(K) + i % K;
         }
         e = cudaMemcpy(m->wmap, map.data(), sizeof(long long) * m->n_params,
                        cudaMemcpyHostToDevice);
@@ -541,7 +664,7 @@ void lbm_mlp_destroy(lbm_mlp *m) {
     cudaFree(m->wb);
     cudaFree(m->wmap);
     for (auto p : m->pre) cudaFree(p);
-    for (auto p : m->act) cudaFree(p);
+    cudaFree(m->act);
     for (auto p : m->actb) cudaFree(p);
     cudaFree(m->g0);
     cudaFree(m->g1);
@@ -549,8 +672,9 @@ void lbm_mlp_destroy(lbm_mlp *m) {
     cudaFree(m->gb1);
     cudaFree(m->loss_part);
     cudaFree(m->tstate);
-    cudaFree(m->xb);
-    cudaFree(m->tb);
+    if (m->fork) cudaEventDestroy(m->fork);
+    if (m->join) cudaEventDestroy(m->join);
+    if (m->cap2) cudaStreamDestroy(m->cap2);
     if (m->cap) cudaStreamDestroy(m->cap);
     delete m;
 }
@@ -565,8 +689,8 @@ lbm_status lbm_mlp_set_params(lbm_mlp *m, const float *host) {
     MCK(m, cudaMemsetAsync(m->v, 0, sizeof(float) * m->n_params, m->stream));
     for (int l = 0; l < m->layers; ++l) {
         const long long nw = (long long)m->widths[l] * m->widths[l + 1];
-        to_bf16<<<grid1(nw), 256, 0, m->stream>>>(m->params + m->w_off[l], m->wb + m->wb_off[l],
-                                                  nw);
+        to_bf16_rows<<<grid1(nw), 256, 0, m->stream>>>(
+            m->params + m->w_off[l], m->wb + m->wb_off[l], m->widths[l + 1], m->widths[l]);
         MCK(m, cudaGetLastError());
     }
     m->steps = 0;
@@ -587,7 +711,7 @@ lbm_status lbm_mlp_forward(lbm_mlp *m, const float *x, int batch, float *y) {
     if (!m || !x || !y) return mfail(m, LBM_EINVAL, "NULL argument");
     if (batch < 1 || batch > m->max_batch) return mfail(m, LBM_EINVAL, "batch out of range");
     MCK(m, forward(m, x, batch, m->stream));
-    MCK(m, cudaMemcpyAsync(y, m->act[m->layers - 1],
+    MCK(m, cudaMemcpyAsync(y, m->act,
                            sizeof(float) * (size_t)batch * m->widths[m->layers],
                            cudaMemcpyDeviceToDevice, m->stream));
     return LBM_OK;
@@ -599,7 +723,9 @@ static lbm_status loss_and_grad(lbm_mlp *m, const float *x, const float *t, int 
                                 double *loss, float *grads_host) {
     cudaStream_t s = m->stream;
     MCK(m, forward(m, x, batch, s));
-    MCK(m, backward(m, t, batch, s));
+    MCK(m, output_grad(m, t, batch, Minibatch{}, s));
+    MCK(m, total_loss(m, batch, s));
+    MCK(m, backward(m, batch, s));
     const long long no = (long long)batch * m->widths[m->layers];
     double hl = 0.0;
     MCK(m, cudaMemcpyAsync(&hl, m->loss_part + 5 * 4096, sizeof(double), cudaMemcpyDeviceToHost,
@@ -649,11 +775,12 @@ lbm_status lbm_mlp_train(lbm_mlp *m, const float *x, const float *t, int n, int 
     const int L = m->layers, kx = m->widths[0], kt = m->widths[L];
     if (!m->tstate) {
         MCK(m, cudaMalloc(&m->tstate, sizeof(TrainState)));
-        MCK(m, cudaMalloc(&m->xb, sizeof(float) * (size_t)m->max_batch * kx));
-        MCK(m, cudaMalloc(&m->tb, sizeof(float) * (size_t)m->max_batch * kt));
-        MCK(m, cudaStreamCreateWithFlags(&m->cap, cudaStreamNonBlocking));
     }
-    TrainState st0{m->steps, 0, 0, 0.f, 0.f, 0.f};
+    if (!m->cap) MCK(m, cudaStreamCreateWithFlags(&m->cap, cudaStreamNonBlocking));
+    if (!m->cap2) MCK(m, cudaStreamCreateWithFlags(&m->cap2, cudaStreamNonBlocking));
+    if (!m->fork) MCK(m, cudaEventCreateWithFlags(&m->fork, cudaEventDisableTiming));
+    if (!m->join) MCK(m, cudaEventCreateWithFlags(&m->join, cudaEventDisableTiming));
+    TrainState st0{m->steps, 0, 0.f, 0.f, 0.f};
     float *hist = nullptr;
     MCK(m, cudaMalloc(&hist, sizeof(float) * (size_t)steps));
     cudaError_t e = cudaMemcpyAsync(m->tstate, &st0, sizeof(st0), cudaMemcpyHostToDevice,
@@ -667,22 +794,25 @@ lbm_status lbm_mlp_train(lbm_mlp *m, const float *x, const float *t, int n, int 
     const float b1 = 0.9f, b2 = 0.999f;
     if (e == cudaSuccess) e = cudaStreamBeginCapture(m->cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaStream_t s = m->cap;
-        cudaError_t le;
-        train_setup<<<1, 1, 0, s>>>(m->tstate, (long long)steps, lr, lr_final, b1, b2);
-        le = cudaGetLastError();
+        cudaStream_t s = m->cap, s2 = m->cap2;
+        const Minibatch mb{m->tstate, seed, n, batch};
+        gather_rows<<<grid1((long long)batch * kx), 256, 0, s>>>(x, kx, mb, m->actb[0]);
+        cudaError_t le = cudaGetLastError();
+        if (le == cudaSuccess) le = forward_layers(m, batch, s);
+        if (le == cudaSuccess) le = output_grad(m, t, batch, mb, s);
+        // beside the backward pass: the step's loss, its scalars and the counters
+        if (le == cudaSuccess) le = cudaEventRecord(m->fork, s);
+        if (le == cudaSuccess) le = cudaStreamWaitEvent(s2, m->fork, 0);
+        if (le == cudaSuccess) le = total_loss(m, batch, s2);
         if (le == cudaSuccess) {
-            gather_rows<<<grid1((long long)batch * (kx > kt ? kx : kt)), 256, 0, s>>>(
-                x, t, n, kx, kt, batch, seed, m->tstate, m->xb, m->tb);
+            train_setup<<<1, 1, 0, s2>>>(m->tstate, (long long)steps, lr, lr_final, b1, b2,
+                                         m->loss_part + 5 * 4096, 1.0 / ((double)batch * kt),
+                                         hist);
             le = cudaGetLastError();
         }
-        if (le == cudaSuccess) le = forward(m, m->xb, batch, s);
-        if (le == cudaSuccess) le = backward(m, m->tb, batch, s);
-        if (le == cudaSuccess) {
-            record_loss<<<1, 1, 0, s>>>(m->loss_part + 5 * 4096,
-                                        1.0 / ((double)batch * kt), m->tstate, hist);
-            le = cudaGetLastError();
-        }
+        if (le == cudaSuccess) le = cudaEventRecord(m->join, s2);
+        if (le == cudaSuccess) le = backward(m, batch, s);
+        if (le == cudaSuccess) le = cudaStreamWaitEvent(s, m->join, 0);
         if (le == cudaSuccess) {
             adam_dev<<<grid1(m->n_params), 256, 0, s>>>(m->params, m->grads, m->m, m->v,
                                                         m->n_params, b1, b2, 1e-8f, m->tstate,
