@@ -555,7 +555,7 @@ lbm_status lbm_mlp_train_step(lbm_mlp *mlp, const float *x, const float *t, int 
  * Adam) is captured once as a CUDA graph and replayed, with no host
  * round trip between steps.  Step s (0-based) draws row j of its minibatch
  * as sample SplitMix64(seed ^ (s batch + j)) mod n (with replacement; all n
- * rows in order when batch >= n) and uses the learning rate
+ * rows in order, again from the first after the last, when batch >= n) and uses the learning rate
  * lr_final + (lr - lr_final)(1 + cos(pi s / steps)) / 2.  The Adam step
  * count carries over between calls.  loss (HOST, `steps` floats, may be
  * NULL) receives each step's loss before its update.  Allocates the

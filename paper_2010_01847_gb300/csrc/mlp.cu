@@ -294,7 +294,7 @@ struct TrainState {
     float lr, c1, c2;     // learning rate and bias corrections of the step
 };
 
-// The minibatch of a training step: row j is sample (batch >= n ? j :
+// The minibatch of a training step: row j is sample (batch >= n ? j mod n :
 // SplitMix64(seed ^ (step batch + j)) mod n), drawn with replacement.
 // st == nullptr: row j is sample j.
 struct Minibatch {
@@ -303,7 +303,8 @@ struct Minibatch {
     int n, batch;
 };
 __device__ __forceinline__ long long sample_of(const Minibatch &mb, long long base, int j) {
-    if (!mb.st || mb.batch >= mb.n) return j;
+    if (!mb.st) return j;
+    if (mb.batch >= mb.n) return j % mb.n;
     return (long long)(splitmix64(mb.seed ^ ((unsigned long long)base + (unsigned)j)) %
                        (unsigned long long)mb.n);
 }

@@ -40,3 +40,22 @@ def test_odd_shapes_match_oracle(widths, batch):
     m = _grad_magnitudes(rp, widths, bf16(x), t)
     bound = len(widths) * 2.0 ** -8 * m + 1e-6 * np.abs(ref_g).max()
     assert (np.abs(g - ref_g) / bound).max() <= 1.0
+
+
+def test_minibatch_larger_than_the_set_repeats_its_rows():
+    """batch > n takes the rows in order, again from the first after the last:
+    the same steps as on a set that holds them so (the loop read rows past the
+    set's end before)."""
+    widths = [3, 16, 24]
+    rng = np.random.default_rng(8)
+    x = rng.uniform(-1, 1, (40, 3)).astype(np.float32)
+    t = rng.normal(0, 1, (40, 24)).astype(np.float32)
+    rows = np.arange(100) % 40
+    out = []
+    for xs, ts in ((x, t), (x[rows], t[rows])):
+        net = plbm.Mlp(widths, max_batch=100)
+        net.init_params(seed=2)
+        loss = net.train(xs, ts, steps=12, batch=100, lr=2e-3, lr_final=1e-3, seed=5)
+        out.append((loss, net.params()))
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    np.testing.assert_array_equal(out[0][1], out[1][1])
