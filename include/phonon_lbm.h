@@ -125,8 +125,8 @@ typedef enum {
     LBM_KERNEL_AUTO = 0,     /* LBM_FP32 up to 5120 nodes (8192 with sides):  */
                              /* resident; LBM_FP64 up to 16384: scalar; from  */
                              /* 2^24 nodes (nx >= 256) wave where it applies  */
-                             /* (FP32: 5 steps per launch, 128-row segments;  */
-                             /* 16-bit: 4 and 256); else vector when nx       */
+                             /* (FP32: 5 steps per launch, 16-bit: 4); else   */
+                             /* vector when nx                                */
                              /* allows, else scalar, and LBM_FP32 lattices in */
                              /* between then take the plain steps of a call   */
                              /* several per launch (tiles of the lattice held */

@@ -367,6 +367,16 @@ bool resident_ok(lbm_ctx *c) {
     return true;
 }
 
+int sm_count(const lbm_ctx *c) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
+        sms < 1) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return sms;
+}
+
 int resolve_kernel(lbm_ctx *c, int requested) {
     const bool vec_ok = c->nx % vector_width(c->precision) == 0;
     // plain 16-bit steps on the vector layout run the pipelined kernel, set
@@ -412,19 +422,18 @@ int resolve_kernel(lbm_ctx *c, int requested) {
     }
     if (requested == KERNEL_AUTO) {
         // without timing (lbm_autotune times them): large lattices the
-        // multi-step kernel where it applies (FP32: 5 steps per launch,
-        // 128-row segments, 424 against 105 GLUPS at 8192^2; 16-bit: 4
-        // steps, 256-row segments, 340 against 171; from 16 M nodes its
-        // strip-segments fill the GPU), else
+        // multi-step kernel where it applies (FP32: 5 steps per launch, 424
+        // against 105 GLUPS at 8192^2; 16-bit: 4 steps, 340 against 171; from
+        // 16 M nodes its strip-segments fill the GPU), else
         // the vector kernel, the fastest single-step
         // kernel measured at 8192^2 for every storage kind (FP32 6.7, 16-bit
         // 6.5 TB/s against the staged kernel's 5.7 and 6.0), with the least
         // set-up for small, launch-latency bound lattices
-        if (c->plane >= WAVE_AUTO_NODES && c->nx >= 256 &&
+        if (c->plane >= WAVE_AUTO_NODES && c->nx >= 256 && sm_count(c) > 0 &&
             wave_supported(c->precision, c->nx, c->ny, c->bc_x, c->bc_y)) {
             const bool fp32 = c->precision == PREC_FP32;
             c->wave_steps = fp32 ? 5 : 4;
-            c->wave_rows = fp32 ? 128 : 256;
+            c->wave_rows = wave_rows(c->precision, c->nx, c->ny, c->wave_steps, sm_count(c));
             return KERNEL_WAVE;
         }
         return vec_ok ? KERNEL_VECTOR : KERNEL_SCALAR;
@@ -448,12 +457,8 @@ void plan_multi(lbm_ctx *c, int requested) {
     if (requested != KERNEL_AUTO || c->precision != PREC_FP32 ||
         (c->kernel != KERNEL_VECTOR && c->kernel != KERNEL_SCALAR))
         return;
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
-        sms < 1) {
-        (void)cudaGetLastError();
-        return;
-    }
+    const int sms = sm_count(c);
+    if (sms < 1) return;
     double best = (c->kernel == KERNEL_VECTOR ? 2.2 : 3.6) + 5.7e-6 * (double)c->plane;
     TilePlan tp;
     const double tile_us = tile_plan(c->nx, c->ny, c->bc_x, c->bc_y, sms, &tp);

@@ -160,6 +160,8 @@ struct WavePlan {
     int steps = 0, rows = 0;
 };
 double wave_plan(int nx, int ny, int sms, WavePlan *out);
+// Rows per segment for a lattice that fills the GPU several times over.
+int wave_rows(int precision, int nx, int ny, int K, int sms);
 bool wave_supported(int precision, int nx, int ny, int bc_x, int bc_y);
 int wave_max_steps(int precision);
 cudaError_t launch_step_wave(int steps, const float *src, float *dst, int nx, int ny, int bc_x,

@@ -48,6 +48,7 @@ constexpr int RING_ELEMS = RING * 8 * 32;  // float2 of one warp's ring
 // the columns a strip with halo H writes
 __host__ __device__ constexpr int halo(int K) { return (K + 1) & ~1; }
 __host__ __device__ constexpr int stride_of(int H) { return 64 - 2 * H; }
+constexpr int HALO16 = 4;                  // 16-bit storage: for every K (wave16.cu)
 
 // One lattice as a strip march sees it: source and destination planes
 // (post-collision, element offset 0 = plane 0, node 0) and segment rows.

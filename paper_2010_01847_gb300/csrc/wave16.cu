@@ -177,7 +177,7 @@ __device__ __forceinline__ void march_step16(March16<K> &m, const Strip16 &a,
 
 // Halo of the 16-bit strips: 4 columns (>= K) for every K, so that the
 // written columns, tx S .. tx S + 55 with S = 56, are whole tiles.
-constexpr int H16 = 4;
+constexpr int H16 = wave::HALO16;
 
 // WALLS = false: y is periodic (the wall rule is left out of the code).
 template <typename T, int K, bool SEAM, bool SR, bool WALLS>
