@@ -69,7 +69,7 @@ struct Product {
 // multiply.  So a stage is 64 deep and STAGES of them are in flight at once:
 // with T = 32 the whole depth of 512 is requested before the first multiply.
 // With one launch per layer and direction, a training step of the
-// 3-256-256-256-256-512 network at 512 rows takes 72 us; a 32-deep loop that
+// 3-256-256-256-256-512 network at 512 rows takes 60 us; a 32-deep loop that
 // loaded, waited and multiplied in turn, in 24 launches, took 207.
 // A row of a tile is padded by 8 elements (an odd number of 16-byte units:
 // ldmatrix reads 8 rows without bank conflicts).
@@ -150,6 +150,25 @@ __device__ __forceinline__ void product_tile(const Product &g, int m0, int n0, u
     constexpr unsigned B_J = 2 * 16 * (B_KMAJOR ? Tile<T>::K_ROW : 1);
     constexpr unsigned A_K = 2 * 16 * (A_KMAJOR ? 1 : Tile<T>::M_ROW);     // next 16 of the depth
     constexpr unsigned B_K = 2 * 16 * (B_KMAJOR ? 1 : Tile<T>::M_ROW);
+    // what the epilogue reads, asked for before the products (behind them each
+    // load would wait for the one before: the stores between may alias)
+    float bias[NJ][2], aux[MI][NJ][4];
+#pragma unroll
+    for (int q = 0; q < NJ; ++q)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int n = n0 + wn + 8 * q + 2 * tg + e;
+            bias[q][e] = g.bias && n < g.N ? g.bias[n] : 0.f;
+#pragma unroll
+            for (int i = 0; i < MI; ++i)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int m = m0 + wm + 16 * i + gr + 8 * h;
+                    aux[i][q][2 * h + e] = g.epi == EPI_GELU_BWD && m < g.M && n < g.N
+                                               ? g.aux[(long long)m * g.N + n]
+                                               : 0.f;
+                }
+        }
     float acc[MI][NJ][4] = {};
     for (int c = 0; c < chunks; ++c) {
         asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
@@ -196,10 +215,10 @@ __device__ __forceinline__ void product_tile(const Product &g, int m0, int n0, u
                 for (int e = 0; e < 2; ++e) {
                     if (n + e >= g.N) continue;
                     const long long o = (long long)m * g.N + n + e;
-                    v[e] = acc[i][q][2 * h + e] + (g.bias ? g.bias[n + e] : 0.f);
+                    v[e] = acc[i][q][2 * h + e] + bias[q][e];
                     if (g.pre) g.pre[o] = v[e];
                     if (g.epi == EPI_GELU) v[e] = gelu(v[e]);
-                    if (g.epi == EPI_GELU_BWD) v[e] = v[e] * gelu_grad(g.aux[o]);
+                    if (g.epi == EPI_GELU_BWD) v[e] = v[e] * gelu_grad(aux[i][q][2 * h + e]);
                     if (g.out) g.out[o] = v[e];
                 }
                 if (g.outb)
@@ -295,52 +314,91 @@ struct TrainState {
 };
 
 // The minibatch of a training step: row j is sample (batch >= n ? j mod n :
-// SplitMix64(seed ^ (step batch + j)) mod n), drawn with replacement.
-// st == nullptr: row j is sample j.
-struct Minibatch {
-    const TrainState *st;
-    unsigned long long seed;
-    int n, batch;
-};
-__device__ __forceinline__ long long sample_of(const Minibatch &mb, long long base, int j) {
-    if (!mb.st) return j;
-    if (mb.batch >= mb.n) return j % mb.n;
-    return (long long)(splitmix64(mb.seed ^ ((unsigned long long)base + (unsigned)j)) %
-                       (unsigned long long)mb.n);
-}
-
-// The step's input rows, in BF16.
-__global__ void gather_rows(const float *__restrict__ x, int kx, Minibatch mb,
-                            __nv_bfloat16 *__restrict__ y) {
-    const long long ld = ld8(kx), total = mb.batch * ld, base = mb.st->local * mb.batch;
+// SplitMix64(seed ^ (step batch + j)) mod n), drawn with replacement.  Writes
+// the samples and their input rows in BF16.
+__global__ void gather_rows(const float *__restrict__ x, int kx, const TrainState *st,
+                            unsigned long long seed, int n, int batch, int *rows,
+                            __nv_bfloat16 *y) {
+    const long long ld = ld8(kx), total = batch * ld;
+    const unsigned long long base = (unsigned long long)st->local * (unsigned long long)batch;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
         const int j = int(i / ld), c = int(i - j * ld);
-        y[i] = __float2bfloat16_rn(c < kx ? x[sample_of(mb, base, j) * kx + c] : 0.f);
+        const int sample = batch >= n ? j % n
+                                      : (int)(splitmix64(seed ^ (base + (unsigned)j)) %
+                                              (unsigned long long)n);
+        if (c == 0) rows[j] = sample;
+        y[i] = __float2bfloat16_rn(c < kx ? x[(long long)sample * kx + c] : 0.f);
     }
 }
 
 // dY = 2 (Y - T) / (B N) (mean squared error), FP32 [B x N] and BF16 (rows of
-// ld8(N)), and the loss partial sums.
-__global__ void mse_grad(const float *__restrict__ y, const float *__restrict__ t, int rows, int N,
-                         Minibatch mb, float scale, float *__restrict__ dy,
-                         __nv_bfloat16 *__restrict__ dyb, double *__restrict__ loss_partials) {
-    const long long n = (long long)rows * N, base = mb.st ? mb.st->local * mb.batch : 0;
+// ld8(N)), and the loss partial sums, one per block.  rows: the sample of each
+// row (nullptr: row j is sample j).  An SM adds about one FP64 value per clock,
+// which bounds this kernel: a thread sums MSE_EACH squares before the block's
+// tree (one value per thread, and the tree over five sums of which four were
+// zero, took 12.8 us at 512 x 512; with the samples drawn again for every
+// element).
+constexpr int MSE_EACH = 4;
+constexpr int LOSS_BLOCKS = 4096;
+unsigned mse_blocks(long long n) {
+    const long long b = (n + 256 * MSE_EACH - 1) / (256 * MSE_EACH);
+    return (unsigned)(b > LOSS_BLOCKS ? LOSS_BLOCKS : b);
+}
+__global__ void __launch_bounds__(256)
+mse_grad(const float *y, const float *t, const int *rows, long long n, int N, float scale,
+         float *dy, __nv_bfloat16 *dyb, double *loss_partials) {
     const int ld = (int)ld8(N);
+    const bool small = n <= 0xffffffffLL;          // 32-bit division
+    auto row_of = [&](long long i) -> long long {
+        return small ? (long long)((unsigned)i / (unsigned)N) : i / N;
+    };
     double s = 0.0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int j = int(i / N), c = int(i - (long long)j * N);
-        const float d = y[i] - t[sample_of(mb, base, j) * N + c];
-        s += (double)(d * d);
-        const float gval = 2.0f * d * scale;
-        dy[i] = gval;
-        dyb[(long long)j * ld + c] = __float2bfloat16_rn(gval);
-        if (c == N - 1)
-            for (int z = N; z < ld; ++z) dyb[(long long)j * ld + z] = __float2bfloat16_rn(0.f);
+    for (long long base = (long long)blockIdx.x * (256 * MSE_EACH); base < n;
+         base += (long long)gridDim.x * (256 * MSE_EACH)) {
+        float d[MSE_EACH];
+#pragma unroll
+        for (int e = 0; e < MSE_EACH; ++e) {
+            const long long i = base + e * 256 + threadIdx.x;
+            d[e] = 0.f;
+            if (i < n) {
+                const long long j = row_of(i);
+                d[e] = y[i] - t[(rows ? (long long)rows[j] : j) * N + (i - j * N)];
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < MSE_EACH; ++e) {
+            const long long i = base + e * 256 + threadIdx.x;
+            if (i >= n) continue;
+            const long long j = row_of(i);
+            const int c = int(i - j * N);
+            s += (double)(d[e] * d[e]);
+            const float gval = 2.0f * d[e] * scale;
+            dy[i] = gval;
+            dyb[j * ld + c] = __float2bfloat16_rn(gval);
+            if (c == N - 1)
+                for (int z = N; z < ld; ++z) dyb[j * ld + z] = __float2bfloat16_rn(0.f);
+        }
     }
-    double acc[5] = {s, 0.0, 0.0, 0.0, 0.0};
-    block_sum5_store(acc, loss_partials + (size_t)blockIdx.x * 5);
+    __shared__ double part[8];
+    const double w = warp_sum_f64(s);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = w;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double sum = 0.0;
+        for (int i = 0; i < 8; ++i) sum += part[i];
+        loss_partials[blockIdx.x] = sum;
+    }
+}
+
+// The total of the loss partial sums in a fixed order (one block).
+__global__ void __launch_bounds__(256)
+sum_loss(const double *partials, int blocks, double *total) {
+    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int b = threadIdx.x; b < blocks; b += 256) acc[0] += partials[b];
+    __shared__ double out[5];
+    block_sum5_store(acc, out);
+    if (threadIdx.x == 0) *total = out[0];
 }
 
 // One Adam update of parameter i (refreshing its BF16 copy if it is a weight).
@@ -428,6 +486,7 @@ struct lbm_mlp {
     // device training loop: state, capture streams (the second takes the
     // step's loss and scalars beside the backward pass) and their events
     TrainState *tstate = nullptr;
+    int *rows = nullptr;                  // the minibatch's samples
     cudaStream_t cap = nullptr, cap2 = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
     double *loss_part = nullptr;
@@ -520,21 +579,21 @@ cudaError_t forward(lbm_mlp *m, const float *x, int batch, cudaStream_t s) {
     return e == cudaSuccess ? forward_layers(m, batch, s) : e;
 }
 
-// dY of the rows the forward pass last ran against targets t (of mb's
-// samples), and the loss partial sums.
-cudaError_t output_grad(lbm_mlp *m, const float *t, int batch, const Minibatch &mb,
-                        cudaStream_t s) {
+// dY of the rows the forward pass last ran against targets t (row j's target
+// is row rows[j] of t; nullptr: row j), and the loss partial sums.
+cudaError_t output_grad(lbm_mlp *m, const float *t, const int *rows, int batch, cudaStream_t s) {
     const int N = m->widths[m->layers];
     const long long no = (long long)batch * N;
-    mse_grad<<<grid1(no), 256, 0, s>>>(m->act, t, batch, N, mb, 1.0f / (float)no, m->g0, m->gb,
-                                       m->loss_part);
+    mse_grad<<<mse_blocks(no), 256, 0, s>>>(m->act, t, rows, no, N, 1.0f / (float)no, m->g0,
+                                            m->gb, m->loss_part);
     return cudaGetLastError();
 }
 
-// The total loss (sum of squares) into loss_part[5 * 4096].
+// The total loss (sum of squares) into loss_part[LOSS_BLOCKS].
 cudaError_t total_loss(lbm_mlp *m, int batch, cudaStream_t s) {
-    return launch_finalize(m->loss_part, (int)grid1((long long)batch * m->widths[m->layers]),
-                           m->loss_part + 5 * 4096, s);
+    sum_loss<<<1, 256, 0, s>>>(m->loss_part, (int)mse_blocks((long long)batch * m->widths[m->layers]),
+                               m->loss_part + LOSS_BLOCKS);
+    return cudaGetLastError();
 }
 
 // Every parameter's gradient (into m->grads) after output_grad, on stream s;
@@ -631,7 +690,8 @@ lbm_status lbm_mlp_create(const int *widths, int n_widths, int max_batch, void *
     al((void **)&m->g1, sizeof(float) * (size_t)max_batch * wmax);
     al((void **)&m->gb, sizeof(__nv_bfloat16) * (size_t)max_batch * ld8(wmax));
     al((void **)&m->gb1, sizeof(__nv_bfloat16) * (size_t)max_batch * ld8(wmax));
-    al((void **)&m->loss_part, sizeof(double) * 5 * 4097);   // partials + total
+    al((void **)&m->loss_part, sizeof(double) * (LOSS_BLOCKS + 1));   // partials + total
+    al((void **)&m->rows, sizeof(int) * (size_t)max_batch);
     if (e == cudaSuccess) {
         std::vector<long long> map(m->n_params, -1);
         for (int l = 0; l < m->layers; ++l) {
@@ -673,6 +733,7 @@ void lbm_mlp_destroy(lbm_mlp *m) {
     cudaFree(m->gb1);
     cudaFree(m->loss_part);
     cudaFree(m->tstate);
+    cudaFree(m->rows);
     if (m->fork) cudaEventDestroy(m->fork);
     if (m->join) cudaEventDestroy(m->join);
     if (m->cap2) cudaStreamDestroy(m->cap2);
@@ -724,12 +785,12 @@ static lbm_status loss_and_grad(lbm_mlp *m, const float *x, const float *t, int 
                                 double *loss, float *grads_host) {
     cudaStream_t s = m->stream;
     MCK(m, forward(m, x, batch, s));
-    MCK(m, output_grad(m, t, batch, Minibatch{}, s));
+    MCK(m, output_grad(m, t, nullptr, batch, s));
     MCK(m, total_loss(m, batch, s));
     MCK(m, backward(m, batch, s));
     const long long no = (long long)batch * m->widths[m->layers];
     double hl = 0.0;
-    MCK(m, cudaMemcpyAsync(&hl, m->loss_part + 5 * 4096, sizeof(double), cudaMemcpyDeviceToHost,
+    MCK(m, cudaMemcpyAsync(&hl, m->loss_part + LOSS_BLOCKS, sizeof(double), cudaMemcpyDeviceToHost,
                            s));
     if (grads_host)
         MCK(m, cudaMemcpyAsync(grads_host, m->grads, sizeof(float) * m->n_params,
@@ -796,18 +857,18 @@ lbm_status lbm_mlp_train(lbm_mlp *m, const float *x, const float *t, int n, int 
     if (e == cudaSuccess) e = cudaStreamBeginCapture(m->cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         cudaStream_t s = m->cap, s2 = m->cap2;
-        const Minibatch mb{m->tstate, seed, n, batch};
-        gather_rows<<<grid1((long long)batch * kx), 256, 0, s>>>(x, kx, mb, m->actb[0]);
+        gather_rows<<<grid1(batch * ld8(kx)), 256, 0, s>>>(x, kx, m->tstate, seed, n, batch,
+                                                           m->rows, m->actb[0]);
         cudaError_t le = cudaGetLastError();
         if (le == cudaSuccess) le = forward_layers(m, batch, s);
-        if (le == cudaSuccess) le = output_grad(m, t, batch, mb, s);
+        if (le == cudaSuccess) le = output_grad(m, t, m->rows, batch, s);
         // beside the backward pass: the step's loss, its scalars and the counters
         if (le == cudaSuccess) le = cudaEventRecord(m->fork, s);
         if (le == cudaSuccess) le = cudaStreamWaitEvent(s2, m->fork, 0);
         if (le == cudaSuccess) le = total_loss(m, batch, s2);
         if (le == cudaSuccess) {
             train_setup<<<1, 1, 0, s2>>>(m->tstate, (long long)steps, lr, lr_final, b1, b2,
-                                         m->loss_part + 5 * 4096, 1.0 / ((double)batch * kt),
+                                         m->loss_part + LOSS_BLOCKS, 1.0 / ((double)batch * kt),
                                          hist);
             le = cudaGetLastError();
         }
