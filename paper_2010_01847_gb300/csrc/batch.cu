@@ -385,13 +385,13 @@ Coef<C> coef_of(const lbm_instance &in, double scale, int precision) {
     const Params p = params_of(in);
     Coef<C> k{};
     k.omega = (C)(1.0 / p.tau);
-    k.sigma = (C)p.sigma;
     k.lambda = (C)p.lambda;
     k.zeta = (C)(p.lambda + p.sigma * p.tau * (1.0 - p.lambda));
     k.w_axis = (C)(2.0 / 9.0);
     k.w_diag = (C)0.25 - k.w_axis;
     k.h_axis = (C)(1.0 / 3.0);
     k.h_diag = ((C)1 - (C)2 * k.h_axis) / (C)4;
+    set_pair_form(k);
     k.u_axis = (C)0.8;
     k.u_diag = ((C)1 - k.u_axis) / (C)2;
     k.jump_axis = (C)(scale * (2.0 / 9.0) * in.bc.delta_e);

@@ -133,7 +133,6 @@ Coef<C> make_coef(const lbm_ctx *c) {
     // Eqs. 13, 15-18, 54 and 58 as the coefficients of lbm_device.cuh.
     Coef<C> k{};
     k.omega = (C)(1.0 / c->tau);
-    k.sigma = (C)c->sigma;
     const double lambda = std::isinf(c->tau_r) ? 0.0 : 1.0 / (2.0 * c->tau_r + 1.0);
     k.lambda = (C)lambda;
     k.zeta = (C)(lambda + c->sigma * c->tau * (1.0 - lambda));
@@ -141,6 +140,7 @@ Coef<C> make_coef(const lbm_ctx *c) {
     k.w_diag = (C)0.25 - k.w_axis;                  // exact: 4 w_axis + 4 w_diag = 1
     k.h_axis = (C)(1.0 / 3.0);
     k.h_diag = ((C)1 - (C)2 * k.h_axis) / (C)4;     // exact: 2 h_axis + 4 h_diag = 1
+    set_pair_form(k);
     k.u_axis = (C)0.8;
     k.u_diag = ((C)1 - k.u_axis) / (C)2;            // exact: u_axis + 2 u_diag = 1
     k.jump_axis = (C)(c->scale * (2.0 / 9.0) * c->delta_e);
