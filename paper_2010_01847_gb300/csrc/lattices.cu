@@ -7,7 +7,8 @@
 // nx*ny*nz, x fastest), deviations d_i = s (e_i - w_i e_ref) with s = 1,
 // pull streaming from the post-collision planes of the previous step, the
 // collision in registers on deviations with exact-sum rounded weights, and
-// captured CUDA graphs of 64 steps.  In a pull step every stored value is
+// captured CUDA graphs of 64 steps (FP32 D3Q14 lattices from half a million
+// nodes: two steps per launch, step2_d3q14).  In a pull step every stored value is
 // read by exactly one node, so one thread per node with x fastest reads each
 // plane row once, coalesced (the +-1 shift along x costs one extra sector
 // per warp, served from L2).
@@ -59,29 +60,47 @@ template <typename C> struct CoefN {
     C h_axis, h_corner;
 };
 
-// The collision of one node, on Q pulled deviations.
+// The collision of one node, on Q pulled deviations.  Opposite velocities
+// (2j, 2j + 1) share their difference, c_i.q and t_i, whose signs alone
+// differ: 108 operations for D3Q14, where population by population they were
+// about 160, with the same roundings.
 template <int LAT, typename C>
 __device__ __forceinline__ void collide_nd(C (&d)[Lat<LAT>::Q], const CoefN<C> &k) {
     using L = Lat<LAT>;
-    C rho = C(0), mx = C(0), my = C(0), mz = C(0);
+    C rho = d[0] + d[1], m[3];
+    bool any[3] = {false, false, false};
 #pragma unroll
     for (int i = 0; i < L::Q; i += 2) {       // opposite velocities are adjacent
-        rho += d[i] + d[i + 1];
-        if (L::cx(i)) mx += L::cx(i) > 0 ? d[i] - d[i + 1] : d[i + 1] - d[i];
-        if (L::cy(i)) my += L::cy(i) > 0 ? d[i] - d[i + 1] : d[i + 1] - d[i];
-        if (L::cz(i)) mz += L::cz(i) > 0 ? d[i] - d[i + 1] : d[i + 1] - d[i];
+        if (i) rho += d[i] + d[i + 1];
+        const C s = d[i] - d[i + 1];
+        const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (!c[a]) continue;
+            m[a] = !any[a] ? (c[a] > 0 ? s : -s) : c[a] > 0 ? m[a] + s : m[a] - s;
+            any[a] = true;
+        }
     }
-    const C qx = mx - k.lambda * mx, qy = my - k.lambda * my, qz = mz - k.lambda * mz;
+    C q[3];
+#pragma unroll
+    for (int a = 0; a < L::DIM; ++a) q[a] = m[a] - k.lambda * m[a];
     const C wa = k.w_axis * rho, wc = k.w_corner * rho;
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
+    for (int i = 0; i < L::Q; i += 2) {
+        const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
         C cq = C(0);
-        if (L::cx(i)) cq += L::cx(i) > 0 ? qx : -qx;
-        if (L::cy(i)) cq += L::cy(i) > 0 ? qy : -qy;
-        if (L::cz(i)) cq += L::cz(i) > 0 ? qz : -qz;
+        bool first = true;
+#pragma unroll
+        for (int a = 0; a < L::DIM; ++a) {
+            if (!c[a]) continue;
+            cq = first ? (c[a] > 0 ? q[a] : -q[a]) : c[a] > 0 ? cq + q[a] : cq - q[a];
+            first = false;
+        }
         const C t = (i < L::AXIS ? k.h_axis : k.h_corner) * cq;
-        const C eq = (i < L::AXIS ? wa : wc) + t;
-        d[i] = d[i] - k.omega * (d[i] - eq) - k.sigma * t;
+        const C w = i < L::AXIS ? wa : wc;
+        const C ep = w + t, em = w - t;
+        d[i] = d[i] - k.omega * (d[i] - ep) - k.sigma * t;
+        d[i + 1] = d[i + 1] - k.omega * (d[i + 1] - em) + k.sigma * t;
     }
 }
 
@@ -91,10 +110,11 @@ struct Dims {
 };
 
 // Pull of the Q populations arriving at node (x, y, z) from the
-// post-collision planes `src` of a periodic lattice.
-template <int LAT, typename T>
-__device__ __forceinline__ void pull_nd(const T *__restrict__ src, const Dims &g, int x, int y,
-                                        int z, typename Store<T>::C (&d)[Lat<LAT>::Q]) {
+// post-collision planes `src` of a periodic lattice.  I: the type of an offset
+// within a plane.
+template <int LAT, typename T, typename I = long long>
+__device__ __forceinline__ void pull_nd(const T *src, const Dims &g, int x, int y, int z,
+                                        typename Store<T>::C (&d)[Lat<LAT>::Q]) {
     using L = Lat<LAT>;
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
@@ -102,24 +122,151 @@ __device__ __forceinline__ void pull_nd(const T *__restrict__ src, const Dims &g
         sx = sx < 0 ? sx + g.nx : (sx >= g.nx ? sx - g.nx : sx);
         sy = sy < 0 ? sy + g.ny : (sy >= g.ny ? sy - g.ny : sy);
         sz = sz < 0 ? sz + g.nz : (sz >= g.nz ? sz - g.nz : sz);
-        d[i] = Store<T>::load(src[(long long)i * g.plane + ((long long)sz * g.ny + sy) * g.nx + sx]);
+        d[i] = Store<T>::load(src[(long long)i * g.plane + (((I)sz * g.ny + sy) * g.nx + sx)]);
     }
 }
 
-template <int LAT, typename T>
+// One step, one thread per node.  I: unsigned for planes of less than 2^31 nodes (the
+// position's four divisions and fourteen offsets in 64 bits were more
+// instructions than the collision), else long long.
+template <int LAT, typename T, typename I>
 __global__ void __launch_bounds__(256)
-step_nd(const T *__restrict__ src, T *__restrict__ dst, Dims g, CoefN<typename Store<T>::C> k) {
+step_nd(const T *src, T *dst, Dims g, CoefN<typename Store<T>::C> k) {
     using C = typename Store<T>::C;
-    const long long node = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (node >= g.plane) return;
-    const int x = int(node % g.nx);
-    const long long r = node / g.nx;
-    const int y = int(r % g.ny), z = int(r / g.ny);
+    const I node = (I)blockIdx.x * blockDim.x + threadIdx.x;
+    if (node >= (I)g.plane) return;
+    const I r = node / (I)g.nx;
+    const int x = int(node - r * (I)g.nx);
+    const int z = int(r / (I)g.ny), y = int(r - (I)z * (I)g.ny);
     C d[Lat<LAT>::Q];
-    pull_nd<LAT, T>(src, g, x, y, z, d);
+    pull_nd<LAT, T, I>(src, g, x, y, z, d);
     collide_nd<LAT>(d, k);
 #pragma unroll
     for (int i = 0; i < Lat<LAT>::Q; ++i) __stcs(dst + (long long)i * g.plane + node, Store<T>::put(d[i]));
+}
+
+// Two time steps of an FP32 D3Q14 lattice per launch.  A single step is bound
+// by memory (112 bytes per node); here a block owns a column of tiles, 32 x 10
+// nodes of (x, y) and planes z0 .. z1 - 1, and marches up z: at position p
+// every thread pulls its node of plane p from the source planes and collides
+// it (step 1, kept in shared memory only), then the inner 30 x 8 threads pull
+// plane p - 1 of step 1 from there, collide again and store step 2.  The outer
+// ring and the planes z0 - 1 and z1 of step 1 are worked out by two blocks.
+// The next plane's loads are issued before step 2 of this one.  The
+// arithmetic is that of step_nd (pull_nd's values, collide_nd).
+// 192^3: 118.0 -> 83.9 us a step; 96^3 15.7 -> 14.4; below PAIR_MIN_NODES
+// single steps are faster (64^3 5.9 against 7.2 us).  It reads and writes 787 MB of DRAM per launch
+// at 192^3, what two steps cannot do without; what is left is each plane's
+// barrier and loads, so several small blocks per SM do better than two large
+// ones: 32 x 16 threads and 2 blocks 95.9 us, 32 x 12 and 3 (spilling) 101.4,
+// 32 x 8 and 4 88.4, 32 x 10 and 3 83.9.
+//
+// Shared memory: the 5 populations with c_z = +1 are pulled two positions
+// after they are written, those with c_z = 0 one, those with c_z = -1 in the
+// same; with one barrier per position a slot may be written again two
+// positions after its last read, so they keep 4, 3 and 2 planes.
+constexpr long long PAIR_MIN_NODES = 1 << 19;
+constexpr int P2_X = 32, P2_Y = 10, P2_THREADS = P2_X * P2_Y, P2_BLOCKS = 3;
+constexpr int P2_SMEM = (5 * 4 + 4 * 3 + 5 * 2) * P2_THREADS * (int)sizeof(float);
+
+__host__ __device__ constexpr int p2_ring(int cz) { return cz > 0 ? 4 : cz == 0 ? 3 : 2; }
+// first element of population i's ring
+__host__ __device__ constexpr int p2_base(int i) {
+    using L = Lat<LBM_LATTICE_D3Q14>;
+    int at = 0;
+    for (int j = 0; j < i; ++j) at += p2_ring(L::cz(j));
+    return at * P2_THREADS;
+}
+
+__global__ void __launch_bounds__(P2_THREADS, P2_BLOCKS)
+step2_d3q14(const float *__restrict__ src, float *__restrict__ dst, Dims g, int tiles_x,
+            int tiles_y, int seg, CoefN<float> k) {
+    using L = Lat<LBM_LATTICE_D3Q14>;
+    extern __shared__ float rings[];
+    const int tx = threadIdx.x % P2_X, ty = threadIdx.x / P2_X;
+    const int by = blockIdx.x / tiles_x % tiles_y, bx = blockIdx.x % tiles_x;
+    const int z0 = int(blockIdx.x / tiles_x / tiles_y) * seg, z1 = min(z0 + seg, g.nz);
+    const int ox = bx * (P2_X - 2) + tx - 1, oy = by * (P2_Y - 2) + ty - 1;
+    const bool own = tx > 0 && tx < P2_X - 1 && ty > 0 && ty < P2_Y - 1 && ox < g.nx && oy < g.ny;
+    auto wrap = [](int v, int n) {
+        v %= n;
+        return v < 0 ? v + n : v;
+    };
+    // byte offsets of the columns and rows the pull reads: [0] c = -1, [1] 0,
+    // [2] +1 (a layer has less than 2^30 nodes; everything else of an address
+    // is the same for the whole block)
+    unsigned xo[3], yo[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        xo[c] = 4u * wrap(ox - (c - 1), g.nx);
+        yo[c] = 4u * ((unsigned)wrap(oy - (c - 1), g.ny) * g.nx);
+    }
+    const long long layer = (long long)g.nx * g.ny;
+    float d[L::Q];
+    // the next plane of step 1 before its collision, from planes zl, zc, zh
+    int zl = wrap(z0 - 2, g.nz), zc = wrap(z0 - 1, g.nz), zh = z0;
+    auto load = [&]() {
+        const float *const z[3] = {src + zh * layer, src + zc * layer, src + zl * layer};
+        zl = zc;
+        zc = zh;
+        zh = zh + 1 == g.nz ? 0 : zh + 1;
+#pragma unroll
+        for (int i = 0; i < L::Q; ++i)
+            d[i] = __ldg(reinterpret_cast<const float *>(
+                reinterpret_cast<const char *>(z[L::cz(i) + 1] + (long long)i * g.plane) +
+                (yo[L::cy(i) + 1] + xo[L::cx(i) + 1])));
+    };
+    load();
+    float *out = dst + (long long)z0 * layer;
+    const unsigned at = own ? 4u * ((unsigned)oy * g.nx + ox) : 0u;
+    int s3 = 0;                            // position mod 3
+    for (int p = z0 - 1, n = 0; p <= z1; ++p, ++n) {
+        collide_nd<LBM_LATTICE_D3Q14>(d, k);
+        float *const mine = rings + threadIdx.x;
+        float *const w4 = mine + (n & 3) * P2_THREADS, *const w3 = mine + s3 * P2_THREADS,
+                    *const w2 = mine + (n & 1) * P2_THREADS;
+#pragma unroll
+        for (int i = 0; i < L::Q; ++i)
+            (L::cz(i) > 0 ? w4 : L::cz(i) == 0 ? w3 : w2)[p2_base(i)] = d[i];
+        __syncthreads();
+        if (p < z1) load();
+        if (n >= 2 && own) {
+            // step 2 of plane p - 1: c_z = +1 from plane p - 2, 0 from p - 1, -1 from p
+            const float *const r4 = mine + ((n + 2) & 3) * P2_THREADS,
+                        *const r3 = mine + (s3 == 0 ? 2 : s3 - 1) * P2_THREADS, *const r2 = w2;
+            float f[L::Q];
+#pragma unroll
+            for (int i = 0; i < L::Q; ++i)
+                f[i] = (L::cz(i) > 0 ? r4 : L::cz(i) == 0 ? r3 : r2)[p2_base(i) - L::cx(i) -
+                                                                     L::cy(i) * P2_X];
+            collide_nd<LBM_LATTICE_D3Q14>(f, k);
+#pragma unroll
+            for (int i = 0; i < L::Q; ++i)
+                __stcs(reinterpret_cast<float *>(
+                           reinterpret_cast<char *>(out + (long long)i * g.plane) + at),
+                       f[i]);
+        }
+        if (n >= 2) out += layer;
+        s3 = s3 == 2 ? 0 : s3 + 1;
+    }
+}
+
+// Blocks' planes: the segments per column that take the fewest rounds of
+// plane positions (P2_BLOCKS blocks per SM; a segment marches 2 planes more than it
+// owns, and its prologue costs about one).
+int p2_segment(const Dims &g, long long tiles, int sms) {
+    int best = g.nz;
+    long long best_cost = -1;
+    for (int s = 1; s <= g.nz; ++s) {
+        const int seg = (g.nz + s - 1) / s;
+        const long long blocks = tiles * ((g.nz + seg - 1) / seg);
+        const long long cost = (blocks + P2_BLOCKS * sms - 1) / (P2_BLOCKS * sms) * (seg + 3);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = seg;
+        }
+    }
+    return best;
 }
 
 // e and q of the state at the current step (pulled when `pulled`, else the
@@ -239,6 +386,17 @@ energy_nd(const T *__restrict__ src, Dims g, bool pulled, double *__restrict__ p
     block_sum5_lane0(acc, partials + (size_t)blockIdx.x * 5);
 }
 
+// Sets bit 0 of *bad if one of the first n values of v is not finite, bit 1 if
+// one of those up to `total` is not.
+__global__ void nonfinite_nd(const double *__restrict__ v, long long n, long long total,
+                             int *__restrict__ bad) {
+    int mine = 0;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += (long long)gridDim.x * blockDim.x)
+        if (!isfinite(v[i])) mine |= i < n ? 1 : 2;
+    if (mine) atomicOr(bad, mine);
+}
+
 constexpr int ENERGY_BLOCKS = 1216;
 
 unsigned grid_of(long long n) {
@@ -299,6 +457,7 @@ struct lbm_nd {
     double *sums = nullptr;         // 5
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     int graph_chunk = 64;
+    int pair_seg = 0;               // planes per block of the two-step kernel; 0: single steps
     std::string err;
 };
 
@@ -354,8 +513,9 @@ template <int LAT, typename T> struct StepNd {
     static cudaError_t run(const lbm_nd *c, int src, cudaStream_t s) {
         using C = typename Store<T>::C;
         const unsigned blocks = (unsigned)((c->g.plane + 255) / 256);
-        step_nd<LAT, T><<<blocks, 256, 0, s>>>((const T *)c->buf[src], (T *)c->buf[1 - src], c->g,
-                                               coef_nd<C>(c));
+        (c->g.plane < 1LL << 31 ? step_nd<LAT, T, unsigned> : step_nd<LAT, T, long long>)
+            <<<blocks, 256, 0, s>>>((const T *)c->buf[src], (T *)c->buf[1 - src], c->g,
+                                    coef_nd<C>(c));
         return cudaGetLastError();
     }
 };
@@ -393,6 +553,36 @@ template <int LAT, typename T> struct EnergyNd {
         return launch_finalize(c->partials, ENERGY_BLOCKS, c->sums, c->stream);
     }
 };
+
+// Two steps from buffer src (FP32 D3Q14).
+cudaError_t nd_launch_pair(const lbm_nd *c, int src, cudaStream_t s) {
+    const int tx = (c->g.nx + P2_X - 3) / (P2_X - 2), ty = (c->g.ny + P2_Y - 3) / (P2_Y - 2);
+    const int segs = (c->g.nz + c->pair_seg - 1) / c->pair_seg;
+    step2_d3q14<<<(unsigned)((long long)tx * ty * segs), P2_THREADS, P2_SMEM, s>>>(
+        (const float *)c->buf[src], (float *)c->buf[1 - src], c->g, tx, ty, c->pair_seg,
+        coef_nd<float>(c));
+    return cudaGetLastError();
+}
+
+// Chooses the two-step kernel where its launches are long enough to pay.
+void nd_plan_pairs(lbm_nd *c) {
+    c->pair_seg = 0;
+    if (c->lattice != LBM_LATTICE_D3Q14 || c->precision != PREC_FP32 ||
+        c->g.plane < PAIR_MIN_NODES || (long long)c->g.nx * c->g.ny >= 1LL << 30)
+        return;
+    const long long tiles = (long long)((c->g.nx + P2_X - 3) / (P2_X - 2)) *
+                            ((c->g.ny + P2_Y - 3) / (P2_Y - 2));
+    if (tiles * c->g.nz > 0x7fffffffLL) return;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
+        sms < 1 ||
+        cudaFuncSetAttribute(step2_d3q14, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM) !=
+            cudaSuccess) {
+        (void)cudaGetLastError();
+        return;
+    }
+    c->pair_seg = p2_segment(c->g, tiles, sms);
+}
 
 void nd_drop_graphs(lbm_nd *c) {
     for (auto &g : c->graph) {
@@ -493,6 +683,7 @@ lbm_status lbm_nd_create(int lattice, int nx, int ny, int nz, double tau_N, doub
         lbm_nd_destroy(c);
         return s;
     }
+    nd_plan_pairs(c);
     *out = c;
     return LBM_OK;
 }
@@ -526,16 +717,21 @@ lbm_status lbm_nd_init(lbm_nd *c, const double *e, const double *q) {
     NdDevice g(c->device);
     if (lbm_status s = nd_scratch(c)) return s;
     const size_t n = (size_t)c->g.plane;
-    for (size_t i = 0; i < n; ++i)
-        if (!std::isfinite(e[i])) return nd_fail(c, LBM_EINVAL, "e is not finite");
-    if (q)
-        for (size_t i = 0; i < n * c->dim; ++i)
-            if (!std::isfinite(q[i])) return nd_fail(c, LBM_EINVAL, "q is not finite");
     NDCK(c, cudaMemcpyAsync(c->fields, e, sizeof(double) * n, cudaMemcpyHostToDevice, c->stream));
     if (q)
         NDCK(c, cudaMemcpyAsync(c->fields + n, q, sizeof(double) * n * c->dim,
                                 cudaMemcpyHostToDevice, c->stream));
-    nd_drop_graphs(c);
+    // captured launches stay valid: nothing in them depends on the fields
+    int *const bad = (int *)c->sums;
+    NDCK(c, cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
+    nonfinite_nd<<<grid_of(c->g.plane), 256, 0, c->stream>>>(
+        c->fields, c->g.plane, q ? c->g.plane * (1 + c->dim) : c->g.plane, bad);
+    NDCK(c, cudaGetLastError());
+    int found = 0;
+    NDCK(c, cudaMemcpyAsync(&found, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    NDCK(c, cudaStreamSynchronize(c->stream));
+    if (found)
+        return nd_fail(c, LBM_EINVAL, found & 1 ? "e is not finite" : "q is not finite");
     NDCK(c, nd_dispatch<InitNd>(c, (const double *)c->fields, q ? (const double *)(c->fields + n)
                                                                 : (const double *)nullptr));
     NDCK(c, cudaStreamSynchronize(c->stream));
@@ -552,6 +748,13 @@ lbm_status lbm_nd_step(lbm_nd *c, long n) {
     if (!c->initialised) return nd_fail(c, LBM_EINVAL, "lbm_nd_init has not been called");
     NdDevice g(c->device);
     long left = n;
+    // two steps per launch, then one or two single steps: the read-outs pull
+    // from the state one step back
+    for (; c->pair_seg > 0 && left > 2; left -= 2) {
+        NDCK(c, nd_launch_pair(c, c->cur, c->stream));
+        c->cur = 1 - c->cur;
+        c->n += 2;
+    }
     if (left >= c->graph_chunk) {
         if (!c->graph[c->cur])
             if (lbm_status s = nd_build_graph(c, c->cur)) return s;
