@@ -128,7 +128,9 @@ __device__ __forceinline__ void pull_nd(const T *src, const Dims &g, int x, int 
     }
 }
 
-// One step, one thread per node.  I: unsigned for planes of less than 2^31 nodes (the
+// One step, one thread per node, in chained launches (small lattices take less
+// time per step than a launch does: D3Q14 32^3 2.25 -> 1.64 us, 64^3
+// 5.86 -> 4.76).  I: unsigned for planes of less than 2^31 nodes (the
 // position's four divisions and fourteen offsets in 64 bits were more
 // instructions than the collision), else long long.
 template <int LAT, typename T, typename I>
@@ -141,7 +143,9 @@ step_nd(const T *src, T *dst, Dims g, CoefN<typename Store<T>::C> k) {
     const int x = int(node - r * (I)g.nx);
     const int z = int(r / (I)g.ny), y = int(r - (I)z * (I)g.ny);
     C d[Lat<LAT>::Q];
+    chain_wait();
     pull_nd<LAT, T, I>(src, g, x, y, z, d);
+    chain_next();
     collide_nd<LAT>(d, k);
 #pragma unroll
     for (int i = 0; i < Lat<LAT>::Q; ++i) __stcs(dst + (long long)i * g.plane + node, Store<T>::put(d[i]));
@@ -157,7 +161,7 @@ step_nd(const T *src, T *dst, Dims g, CoefN<typename Store<T>::C> k) {
 // The next plane's loads are issued before step 2 of this one.  The
 // arithmetic is that of step_nd (pull_nd's values, collide_nd).
 // 192^3: 118.0 -> 83.9 us a step; 96^3 15.7 -> 14.4; below PAIR_MIN_NODES
-// single steps are faster (64^3 5.9 against 7.2 us).  It reads and writes 787 MB of DRAM per launch
+// chained single steps are faster (80^3 8.1 against 9.3 us, 64^3 4.8 against 7.2).  It reads and writes 787 MB of DRAM per launch
 // at 192^3, what two steps cannot do without; what is left is each plane's
 // barrier and loads, so several small blocks per SM do better than two large
 // ones: 32 x 16 threads and 2 blocks 95.9 us, 32 x 12 and 3 (spilling) 101.4,
@@ -527,10 +531,10 @@ template <int LAT, typename T> struct StepNd {
     static cudaError_t run(const lbm_nd *c, int src, cudaStream_t s) {
         using C = typename Store<T>::C;
         const unsigned blocks = (unsigned)((c->g.plane + 255) / 256);
-        (c->g.plane < 1LL << 31 ? step_nd<LAT, T, unsigned> : step_nd<LAT, T, long long>)
-            <<<blocks, 256, 0, s>>>((const T *)c->buf[src], (T *)c->buf[1 - src], c->g,
-                                    coef_nd<C>(c));
-        return cudaGetLastError();
+        return launch_chained(c->g.plane < 1LL << 31 ? step_nd<LAT, T, unsigned>
+                                                     : step_nd<LAT, T, long long>,
+                              blocks, 256, 0, s, (const T *)c->buf[src], (T *)c->buf[1 - src],
+                              c->g, coef_nd<C>(c));
     }
 };
 template <int LAT, typename T> struct InitNd {

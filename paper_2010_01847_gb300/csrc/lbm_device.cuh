@@ -79,6 +79,18 @@ template <typename C> inline void set_pair_form(Coef<C> &k) {
     k.h2_diag = (C)2 * k.h_diag;
 }
 
+// Launches of a chain (launch_chained): chain_wait before anything that the
+// launch before writes is read or that it reads is written, then chain_next
+// once this block's own reads are issued, so that the next launch's blocks are
+// in place when this one ends.  (After the wait: never more than two launches
+// of a chain overlap.)  No effect in other launches.
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void chain_next() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Storage traits: how a population plane element is stored and converted.
 template <typename T> struct Store;
 template <> struct Store<float> {

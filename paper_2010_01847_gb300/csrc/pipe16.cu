@@ -98,7 +98,7 @@ __device__ __forceinline__ VPos vpos(long long t, long long total, int tpr, int 
 
 template <typename T, bool SR>
 __global__ void __launch_bounds__(THREADS, PLBM_P16_BLOCKS)
-step_pipe16(const T *__restrict__ src, T *__restrict__ dst, int nx, int ny, long long plane,
+step_pipe16(const T *src, T *dst, int nx, int ny, long long plane,
             int bc_x, int bc_y, Coef<float> k) {
     extern __shared__ uint4 slots[];        // [STAGES][SLOTS][THREADS]
     const int tid = threadIdx.x, lane = tid & 31;
@@ -157,6 +157,7 @@ step_pipe16(const T *__restrict__ src, T *__restrict__ dst, int nx, int ny, long
     const long long stride = gridDim.x;
     // prologue: the first STAGES vectors in flight, one copy group each
     VPos cur = vpos(c * THREADS + tid, total, tpr, ny, walls, lane);
+    chain_wait();
     issue(cur, 0);
     cp_async_commit();
 #pragma unroll
@@ -165,6 +166,7 @@ step_pipe16(const T *__restrict__ src, T *__restrict__ dst, int nx, int ny, long
         if (cs < chunks) issue(vpos(cs * THREADS + tid, total, tpr, ny, walls, lane), s);
         cp_async_commit();
     }
+    chain_next();       // its blocks take the places of this launch's as they end
     int st = 0;
     for (; c < chunks; c += stride) {
         const long long t = c * THREADS + tid;
@@ -303,13 +305,8 @@ cudaError_t launch_step_pipe16(const T *src, T *dst, int nx, int ny, int bc_x, i
     if (!p.ready) return cudaErrorNotReady;      // prepare_pipe16 was not called on this device
     const long long chunks = ((long long)(nx / 8) * ny + THREADS - 1) / THREADS;
     const int grid = (int)(chunks < p.grid ? chunks : p.grid);
-    if (sr)
-        step_pipe16<T, true><<<grid, THREADS, SMEM, stream>>>(src, dst, nx, ny,
-                                                              (long long)nx * ny, bc_x, bc_y, k);
-    else
-        step_pipe16<T, false><<<grid, THREADS, SMEM, stream>>>(src, dst, nx, ny,
-                                                               (long long)nx * ny, bc_x, bc_y, k);
-    return cudaGetLastError();
+    return launch_chained(sr ? step_pipe16<T, true> : step_pipe16<T, false>, grid, THREADS, SMEM,
+                          stream, src, dst, nx, ny, (long long)nx * ny, bc_x, bc_y, k);
 }
 
 template cudaError_t launch_step_pipe16<__half>(const __half *, __half *, int, int, int, int,
