@@ -632,9 +632,10 @@ def run_d3q14(args):
                    "l2": "inputs larger than L2; no flush"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": None,
-                     "peak_source": peak_kind, "kernel": "step_nd",
+                     "peak_source": peak_kind,
+                     "kernel": "step2_d3q14" if pairs else "step_nd",
                      "bytes_per_site_update": bps},
-        "clocks": sampler.summary(), "gpu_launches": args.steps, "e2e": None,
+        "clocks": sampler.summary(), "gpu_launches": launches, "e2e": None,
         "cpu_baseline": None, "energy_drift": drift,
     }
     print(json.dumps(line), flush=True)
