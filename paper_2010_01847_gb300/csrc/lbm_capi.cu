@@ -1206,6 +1206,12 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
             for (int ks : {2, 3, 4})
                 for (int rows : {128, 256}) cands[nc++] = {KERNEL_WAVE, ks, rows};
         }
+        // and the shape LBM_KERNEL_AUTO runs from this size
+        if (c->plane >= WAVE_AUTO_NODES && c->nx >= 256 && sm_count(c) > 0) {
+            const int ks = c->precision == PREC_FP32 ? 5 : 4;
+            cands[nc++] = {KERNEL_WAVE, ks,
+                           wave_rows(c->precision, c->nx, c->ny, ks, sm_count(c))};
+        }
     }
 
     for (int i = 0; i < nc; ++i) cands[i].multi = MULTI_NONE;
@@ -1215,7 +1221,10 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
         c->kernel = cands[0].kernel;
         plan_multi(c, KERNEL_AUTO);
         c->kernel = k0;
-        if (c->multi != MULTI_NONE) cands[nc++] = {cands[0].kernel, 0, 0, c->multi};
+        // (from 16 M nodes the strip march is among the wave candidates)
+        if (c->multi == MULTI_TILE ||
+            (c->multi == MULTI_WAVE && (c->plane < WAVE_AUTO_NODES || c->nx < 256)))
+            cands[nc++] = {cands[0].kernel, 0, 0, c->multi};
     }
     const int tuned_multi = c->multi;
 
