@@ -59,6 +59,8 @@ struct lbm_ctx {
     long long timed_launches[3] = {0, 0, 0}, timed_steps[3] = {0, 0, 0};
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
+    // what the launches in `graph` were captured with (see current_graphs)
+    struct Captured { int kernel = -1, wave_steps = 0, wave_rows = 0; StagedPlan plan; } captured;
     void *prev = nullptr;       // residual history, 3 planes of the compute type
     bool have_prev = false;
     long prev_step = 0;
@@ -642,6 +644,28 @@ int wave_graph_launches(const lbm_ctx *c) {
     return 2 * (pairs > 1 ? pairs : 1);
 }
 
+// Drops the captured launches if another kernel or shape has been selected
+// since the capture: a replay advances the lattice by the steps it was captured
+// with, and the callers count those of the current selection.  Checked here, at
+// the one place that replays, because the selection changes in several
+// (resolve_kernel takes its own steps per launch and rows for AUTO).
+void current_graphs(lbm_ctx *c) {
+    const lbm_ctx::Captured &g = c->captured;
+    bool same = g.kernel == c->kernel;
+    if (c->kernel == KERNEL_WAVE)
+        same = same && g.wave_steps == c->wave_steps && g.wave_rows == c->wave_rows;
+    if (c->kernel == KERNEL_STAGED)
+        same = same && g.plan.stages == c->plan.stages &&
+               g.plan.ctas_per_sm == c->plan.ctas_per_sm && g.plan.grid == c->plan.grid &&
+               g.plan.consumer_warps == c->plan.consumer_warps && g.plan.hint == c->plan.hint;
+    if (same) return;
+    drop_graphs(c);
+    c->captured.kernel = c->kernel;
+    c->captured.wave_steps = c->wave_steps;
+    c->captured.wave_rows = c->wave_rows;
+    c->captured.plan = c->plan;
+}
+
 lbm_status build_graph(lbm_ctx *c, int start) {
     CK(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     int src = start;
@@ -776,6 +800,7 @@ lbm_status advance(lbm_ctx *c, long n, bool end_readable) {
         const int K = c->wave_steps;
         const int gl = wave_graph_launches(c);
         if (!c->timing && c->graph_chunk > 0 && m >= (long)gl * K) {
+            current_graphs(c);
             if (!c->graph[c->cur])
                 if (lbm_status s = build_graph(c, c->cur)) return s;
             while (m >= (long)gl * K) {      // an even number of launches: cur unchanged
@@ -802,6 +827,7 @@ lbm_status advance(lbm_ctx *c, long n, bool end_readable) {
     }
     long left = n;
     if (!c->timing && c->graph_chunk > 0 && left >= c->graph_chunk) {
+        current_graphs(c);
         if (!c->graph[c->cur])
             if (lbm_status s = build_graph(c, c->cur)) return s;
         while (left >= c->graph_chunk) {
