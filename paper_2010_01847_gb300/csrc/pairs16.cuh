@@ -11,6 +11,8 @@
 // live than unpacking all 8 nodes first.
 #pragma once
 
+#include <type_traits>
+
 #include "refs16.cuh"
 
 namespace plbm {
@@ -111,10 +113,22 @@ __device__ __forceinline__ void collide_words16(uint4 (&w)[8], const Coef<float>
         if (m == 2) { r23 = rho; x23 = mx; y23 = my; }
         if (m == 3) { r23 = f_add(r23, rho); x23 = f_add(x23, mx); y23 = f_add(y23, my); }
         relax_f32<float2, false>(f, rho, mx, my, k);
+        // (in BF16 the differences take the populations' registers; in FP16 they
+        // are formed again for each word: the other way round 68 and 24 bytes
+        // are spilled, 2048^2 stochastic 37.8 us against 37.15, 34.5 against 33.6)
+        auto less = [&](int i) { return f_sub(f[i], make_float2(Re[i], Re[i])); };
+        if constexpr (!std::is_same<T, __half>::value) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) f[i] = less(i);
+        }
+        auto stored = [&](int i) {
+            if constexpr (std::is_same<T, __half>::value) return less(i);
+            else return f[i];
+        };
+        const unsigned mask = sr_mask<SR>(stored(0), stored(1));
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-            set_word(w[i], m,
-                     store_word<T, SR>(f_sub(f[i], make_float2(Re[i], Re[i])), pair0 + m, i));
+            set_word(w[i], m, store_word<T, SR>(stored(i), pair0 + m, i, mask));
     }
     sums[0] = tile_tree_pairs(r01, r23);
     sums[1] = tile_tree_pairs(x01, x23);

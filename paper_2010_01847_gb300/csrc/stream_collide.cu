@@ -75,12 +75,17 @@ step_scalar16(const T *__restrict__ src, T *__restrict__ dst, int nx, int ny, lo
     // stochastic rounding both lanes of a pair form the pair's random bits
     // (lane parity = node parity: blocks hold whole warps)
     const bool odd = node & 1;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    auto stored = [&](int i) {
         const float v = f_sub(d[i], Re[i]);
         const float o = SR ? __shfl_xor_sync(0xffffffffu, v, 1) : 0.f;
-        const unsigned wd = store_word<T, SR>(odd ? make_float2(o, v) : make_float2(v, o),
-                                              (unsigned)(node >> 1), i);
+        return odd ? make_float2(o, v) : make_float2(v, o);
+    };
+    const float2 v0 = stored(0), v1 = stored(1);
+    const unsigned mask = sr_mask<SR>(v0, v1);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const unsigned wd = store_word<T, SR>(i == 0 ? v0 : i == 1 ? v1 : stored(i),
+                                              (unsigned)(node >> 1), i, mask);
         if (valid)
             reinterpret_cast<unsigned short *>(dst)[(long long)i * plane + node] =
                 (unsigned short)(odd ? wd >> 16 : wd & 0xffffu);

@@ -291,14 +291,19 @@ __device__ __forceinline__ void collide_store16(float (&n)[8][8], const Coef<flo
         relax_f32(n[j], rho[j], mx[j], my[j], k);
     }
     ref_pops(ref_of<T>(enc), k, Re);
+    // node pairs (2m, 2m + 1), as the pair kernels
+    auto stored = [&](int m, int i) {
+        return make_float2(f_sub(n[2 * m][i], Re[i]), f_sub(n[2 * m + 1][i], Re[i]));
+    };
+    unsigned mask[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) mask[m] = sr_mask<SR>(stored(m, 0), stored(m, 1));
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         unsigned wd[4];
 #pragma unroll
-        for (int m = 0; m < 4; ++m)       // node pairs (2m, 2m + 1), as the pair kernels
-            wd[m] = store_word<T, SR>(
-                make_float2(f_sub(n[2 * m][i], Re[i]), f_sub(n[2 * m + 1][i], Re[i])),
-                (unsigned)(out >> 1) + m, i);
+        for (int m = 0; m < 4; ++m)
+            wd[m] = store_word<T, SR>(stored(m, i), (unsigned)(out >> 1) + m, i, mask[m]);
         st_stream(dst + (long long)i * plane + out, make_uint4(wd[0], wd[1], wd[2], wd[3]));
     }
     st_ref(dst, k, tile, enc,

@@ -162,10 +162,12 @@ __device__ __forceinline__ void march_step16(March16<K> &m, const Strip16 &a,
                 const long long node = (long long)r * a.nx + xa;
                 T *o = (T *)a.dst + node;
 #pragma unroll
+                for (int i = 0; i < 8; ++i) d[i] = f_sub(d[i], make_float2(Re[i], Re[i]));
+                const unsigned mask = sr_mask<SR>(d[0], d[1]);
+#pragma unroll
                 for (int i = 0; i < 8; ++i)
                     st_word(o + (long long)i * a.plane,
-                            store_word<T, SR>(f_sub(d[i], make_float2(Re[i], Re[i])),
-                                              (unsigned)(node >> 1), i));
+                            store_word<T, SR>(d[i], (unsigned)(node >> 1), i, mask));
                 if (rec_lane)
                     st_rec((T *)a.dst + ref_at(k, (long long)r * k.tiles_x + (xa >> 3)),
                            make_uint4(m.enc.x, m.enc.y, nxt.x, nxt.y));
