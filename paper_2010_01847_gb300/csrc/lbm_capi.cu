@@ -17,6 +17,14 @@ using namespace plbm;
 
 enum { MULTI_NONE = 0, MULTI_TILE = 1, MULTI_WAVE = 2 };
 
+// The multi-step kernel of a mid-size lattice and its shape.
+struct Multi {
+    int kind = MULTI_NONE;
+    TilePlan tile;
+    WavePlan wave;
+    int steps() const { return kind == MULTI_TILE ? tile.steps : wave.steps; }
+};
+
 struct lbm_ctx {
     int device = 0;
     int nx = 0, ny = 0;
@@ -47,9 +55,7 @@ struct lbm_ctx {
     int wave_rows = 128;        // and rows per strip segment
     // multi-step launches of lattices whose single steps run on `kernel`
     // (mid sizes, chosen by size or by lbm_autotune)
-    int multi = MULTI_NONE;
-    TilePlan tile;
-    WavePlan wplan;
+    Multi multi;
     int graph_chunk = 64;
     // launch timing (lbm_set_launch_timing): event pairs around launches
     bool timing = false;
@@ -454,28 +460,28 @@ int resolve_kernel(lbm_ctx *c, int requested) {
 // / 3.6, 1024^2 4.5 (wave) / 8.3, 2048^2 13.0 (wave) / 44, 2001^2 square 29.8
 // / 81.8; a single step costs 2.2-3.7 us plus about 6 us per 2^20 nodes in
 // L2 (10.5 beyond it).
-void plan_multi(lbm_ctx *c, int requested) {
-    c->multi = MULTI_NONE;
-    if (requested != KERNEL_AUTO || c->precision != PREC_FP32 ||
-        (c->kernel != KERNEL_VECTOR && c->kernel != KERNEL_SCALAR))
-        return;
+// `kernel`: that of the lattice's single steps.
+Multi plan_multi(const lbm_ctx *c, int kernel) {
+    Multi m;
+    if (c->precision != PREC_FP32 || (kernel != KERNEL_VECTOR && kernel != KERNEL_SCALAR)) return m;
     const int sms = sm_count(c);
-    if (sms < 1) return;
-    double best = (c->kernel == KERNEL_VECTOR ? 2.2 : 3.6) + 5.7e-6 * (double)c->plane;
+    if (sms < 1) return m;
+    double best = (kernel == KERNEL_VECTOR ? 2.2 : 3.6) + 5.7e-6 * (double)c->plane;
     TilePlan tp;
     const double tile_us = tile_plan(c->nx, c->ny, c->bc_x, c->bc_y, sms, &tp);
     if (tp.steps > 0 && tile_us < 0.9 * best) {
-        c->multi = MULTI_TILE;
-        c->tile = tp;
+        m.kind = MULTI_TILE;
+        m.tile = tp;
         best = tile_us;
     }
-    if (!wave_supported(c->precision, c->nx, c->ny, c->bc_x, c->bc_y)) return;
+    if (!wave_supported(c->precision, c->nx, c->ny, c->bc_x, c->bc_y)) return m;
     WavePlan wp;
     const double wave_us = wave_plan(c->nx, c->ny, sms, &wp);
     if (wave_us < best) {
-        c->multi = MULTI_WAVE;
-        c->wplan = wp;
+        m.kind = MULTI_WAVE;
+        m.wave = wp;
     }
+    return m;
 }
 
 lbm_status create_common(lbm_grid g, double tau_N, double tau_R, lbm_boundary bc,
@@ -569,7 +575,7 @@ lbm_status create_common(lbm_grid g, double tau_N, double tau_R, lbm_boundary bc
         return s;
     }
     c->kernel = resolve_kernel(c, KERNEL_AUTO);
-    plan_multi(c, KERNEL_AUTO);
+    c->multi = plan_multi(c, c->kernel);
     *out = c;
     return LBM_OK;
 }
@@ -626,15 +632,15 @@ cudaError_t wave_launch(const lbm_ctx *c, int src, int steps, cudaStream_t s) {
                               c->bc_x, c->bc_y, make_coef<float>(c), c->wave_rows, s);
 }
 
-// One launch of `steps` steps of the context's mid-size multi-step kernel
-// (FP32) from buffer src.
-cudaError_t multi_launch(const lbm_ctx *c, int src, int steps, cudaStream_t s) {
+// One launch of `steps` steps of a mid-size multi-step kernel (FP32) from
+// buffer src.
+cudaError_t multi_launch(const lbm_ctx *c, const Multi &m, int src, int steps, cudaStream_t s) {
     const float *in = (const float *)c->buf[src];
     float *out = (float *)c->buf[1 - src];
     const Coef<float> k = make_coef<float>(c);
-    if (c->multi == MULTI_TILE)
-        return launch_tile(c->tile, steps, in, out, c->nx, c->ny, c->bc_x, c->bc_y, k, s);
-    return launch_step_wave(steps, in, out, c->nx, c->ny, c->bc_x, c->bc_y, k, c->wplan.rows, s);
+    if (m.kind == MULTI_TILE)
+        return launch_tile(m.tile, steps, in, out, c->nx, c->ny, c->bc_x, c->bc_y, k, s);
+    return launch_step_wave(steps, in, out, c->nx, c->ny, c->bc_x, c->bc_y, k, m.wave.rows, s);
 }
 
 // Launches in one captured graph of multi-step launches: an even number (the
@@ -773,17 +779,17 @@ lbm_status advance(lbm_ctx *c, long n, bool end_readable) {
         c->launches += 1;
         return LBM_OK;
     }
-    if (c->multi != MULTI_NONE) {
+    if (c->multi.kind != MULTI_NONE) {
         // launched directly: a launch takes longer than its submission, and a
         // captured graph would have to be built again after every lbm_init
         const long tail = end_readable ? 1 : 0;
-        const int K = c->multi == MULTI_TILE ? c->tile.steps : c->wplan.steps;
+        const int K = c->multi.steps();
         long m = n - tail;
-        while (m >= (c->multi == MULTI_TILE ? 1 : WAVE_MIN_STEPS)) {
+        while (m >= (c->multi.kind == MULTI_TILE ? 1 : WAVE_MIN_STEPS)) {
             const int k = m >= K ? K : (int)m;
             int slot;
             CK(c, timed_begin(c, TIMED_WAVE, k, &slot));
-            CK(c, multi_launch(c, c->cur, k, c->stream));
+            CK(c, multi_launch(c, c->multi, c->cur, k, c->stream));
             CK(c, timed_end(c, slot));
             c->cur = 1 - c->cur;
             m -= k;
@@ -1105,7 +1111,7 @@ lbm_status lbm_set_kernel(lbm_ctx *c, int kernel) {
         drop_graphs(c);
         c->kernel = k;
     }
-    plan_multi(c, kernel);
+    c->multi = kernel == KERNEL_AUTO ? plan_multi(c, k) : Multi();
     return LBM_OK;
 }
 
@@ -1213,7 +1219,7 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
     if (lbm_status s = ensure_scratch(c, false)) return s;   // the status word
     // wave: stages = steps, cw = segment rows; multi: the mid-size multi-step
     // kernel the lattice's size picks, its single steps on `kernel`
-    struct Cand { int kernel, stages, cw, multi; };
+    struct Cand { int kernel, stages, cw; bool multi; };
     Cand cands[17];
     int nc = 0;
     const bool sides = has_sides(c);      // the per-side rules: scalar and vector kernels
@@ -1240,19 +1246,12 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
         }
     }
 
-    for (int i = 0; i < nc; ++i) cands[i].multi = MULTI_NONE;
-    const int old_multi = c->multi;
-    if (cands[0].kernel == KERNEL_VECTOR || cands[0].kernel == KERNEL_SCALAR) {
-        const int k0 = c->kernel;
-        c->kernel = cands[0].kernel;
-        plan_multi(c, KERNEL_AUTO);
-        c->kernel = k0;
-        // (from 16 M nodes the strip march is among the wave candidates)
-        if (c->multi == MULTI_TILE ||
-            (c->multi == MULTI_WAVE && (c->plane < WAVE_AUTO_NODES || c->nx < 256)))
-            cands[nc++] = {cands[0].kernel, 0, 0, c->multi};
-    }
-    const int tuned_multi = c->multi;
+    for (int i = 0; i < nc; ++i) cands[i].multi = false;
+    const Multi multi = plan_multi(c, cands[0].kernel);
+    // (from 16 M nodes the strip march is among the wave candidates)
+    if (multi.kind == MULTI_TILE ||
+        (multi.kind == MULTI_WAVE && (c->plane < WAVE_AUTO_NODES || c->nx < 256)))
+        cands[nc++] = {cands[0].kernel, 0, 0, true};
 
     // keep the state: copy both buffers aside when the lattice holds one
     void *saved = nullptr;
@@ -1262,6 +1261,8 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
             CK(c, cudaMemcpyAsync((char *)saved + i * c->buf_bytes, c->buf[i], c->buf_bytes,
                                   cudaMemcpyDeviceToDevice, c->stream));
     }
+    // (the candidates run with the context's kernel and shapes set to theirs;
+    // whatever fails below leaves the selection as it was)
     const int old_kernel = c->kernel;
     const StagedPlan old_plan = c->plan;
     const int old_ws = c->wave_steps, old_wr = c->wave_rows;
@@ -1281,16 +1282,16 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
         c->kernel = cands[i].kernel;
         c->plan = p;
         long steps_timed = trial_steps;
-        if (cands[i].multi != MULTI_NONE) {
-            const int K = tuned_multi == MULTI_TILE ? c->tile.steps : c->wplan.steps;
+        if (cands[i].multi) {
+            const int K = multi.steps();
             int launches = (trial_steps + K - 1) / K;
             launches += launches & 1;
             steps_timed = (long)launches * K;
             for (int s = 0; s < 2 && err == cudaSuccess; ++s)      // warm-up
-                err = multi_launch(c, s & 1, K, c->stream);
+                err = multi_launch(c, multi, s & 1, K, c->stream);
             if (err == cudaSuccess) err = cudaEventRecord(e0, c->stream);
             for (int s = 0; s < launches && err == cudaSuccess; ++s)
-                err = multi_launch(c, s & 1, K, c->stream);
+                err = multi_launch(c, multi, s & 1, K, c->stream);
         } else if (c->kernel == KERNEL_WAVE) {
             // its point is several steps per launch: time whole launches, an
             // even number (the buffers end where they began)
@@ -1332,6 +1333,8 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
             best_plan = p;
         }
     }
+    c->kernel = old_kernel;
+    c->plan = old_plan;
     c->wave_steps = old_ws;
     c->wave_rows = old_wr;
     if (e0) cudaEventDestroy(e0);
@@ -1343,20 +1346,13 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
         cudaFreeAsync(saved, c->stream);
     }
     if (err == cudaSuccess) err = cudaStreamSynchronize(c->stream);
-    if (err != cudaSuccess || best_i < 0) {
-        c->kernel = old_kernel;
-        c->plan = old_plan;
-        c->multi = old_multi;
-        c->wave_steps = old_ws;
-        c->wave_rows = old_wr;
-        return err != cudaSuccess ? cuda_fail(c, err, "lbm_autotune")
-                                  : fail(c, LBM_ECUDA, "no kernel could be timed");
-    }
+    if (err != cudaSuccess) return cuda_fail(c, err, "lbm_autotune");
+    if (best_i < 0) return fail(c, LBM_ECUDA, "no kernel could be timed");
     if (lbm_status s = check_status(c)) return s;
     drop_graphs(c);
     c->kernel = cands[best_i].kernel;
     c->plan = best_plan;
-    c->multi = cands[best_i].multi;
+    c->multi = cands[best_i].multi ? multi : Multi();
     if (cands[best_i].kernel == KERNEL_WAVE) {
         c->wave_steps = cands[best_i].stages;
         c->wave_rows = cands[best_i].cw;
