@@ -607,16 +607,16 @@ def run_d3q14(args):
     sampler = ClockSampler(dev.index)
     with sampler:
         t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        launches = lat.kernel_launches
         t0.record(stream)
         lat.step(args.steps)
         t1.record(stream)
         torch.cuda.synchronize()
+        launches = lat.kernel_launches - launches
     elapsed = t0.elapsed_time(t1) / 1e3
     sites = n ** 3
-    # FP32 lattices of this size take two steps per launch (one read and one
-    # write of the state for both) until one or two single steps are left
-    pairs = (args.steps - 1) // 2 if prec == "fp32" and sites >= 1 << 19 else 0
-    launches = args.steps - pairs
+    # one read and one write of the state per launch, of one or two steps
+    pairs = args.steps - launches
     bps = 2 * 14 * STORAGE_BYTES[prec] * launches / args.steps
     achieved = bps * sites * args.steps / elapsed / 1e9
     peak, peak_kind = measured_peak()

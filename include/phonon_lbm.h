@@ -697,6 +697,10 @@ lbm_status lbm_nd_populations(lbm_nd *ctx, double *f);
 lbm_status lbm_nd_energy(lbm_nd *ctx, double *total);
 
 long lbm_nd_step_count(const lbm_nd *ctx);
+
+/* Number of stream-collide kernel launches queued since lbm_nd_init (a launch
+ * of two steps counts once). */
+long long lbm_nd_kernel_launches(const lbm_nd *ctx);
 void lbm_nd_destroy(lbm_nd *ctx);
 const char *lbm_nd_last_error(const lbm_nd *ctx);
 

@@ -60,7 +60,7 @@ EXPORTS = [
     "lbm_residual_noalloc", "lbm_check_bounded_wait", "lbm_probe_resident_wait",
     "lbm_nd_lattice_speed", "lbm_nd_create", "lbm_nd_init", "lbm_nd_step", "lbm_nd_sync",
     "lbm_nd_moments", "lbm_nd_populations", "lbm_nd_energy", "lbm_nd_step_count",
-    "lbm_nd_destroy", "lbm_nd_last_error",
+    "lbm_nd_kernel_launches", "lbm_nd_destroy", "lbm_nd_last_error",
 ]
 NOALLOC_MAX_NODES = 16777216
 
@@ -188,6 +188,7 @@ def load_library(path: str = LIB_PATH):
         "lbm_nd_populations": (st, [vp, dp]),
         "lbm_nd_energy": (st, [vp, dp]),
         "lbm_nd_step_count": (c_long, [vp]),
+        "lbm_nd_kernel_launches": (ctypes.c_longlong, [vp]),
         "lbm_nd_destroy": (None, [vp]),
         "lbm_nd_last_error": (ctypes.c_char_p, [vp]),
     }
@@ -863,3 +864,7 @@ class LatticeND:
     @property
     def step_count(self) -> int:
         return self._lib.lbm_nd_step_count(self._ctx)
+
+    @property
+    def kernel_launches(self) -> int:
+        return self._lib.lbm_nd_kernel_launches(self._ctx)

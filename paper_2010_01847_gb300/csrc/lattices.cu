@@ -457,6 +457,7 @@ struct lbm_nd {
     size_t buf_bytes = 0;
     int cur = 0;
     long n = 0;
+    long long launches = 0;         // stream-collide launches since lbm_nd_init
     bool initialised = false;
     double *fields = nullptr;       // (1 + dim) planes of doubles
     double *partials = nullptr;     // ENERGY_BLOCKS x 5
@@ -755,6 +756,7 @@ lbm_status lbm_nd_init(lbm_nd *c, const double *e, const double *q) {
     NDCK(c, cudaStreamSynchronize(c->stream));
     c->cur = 0;
     c->n = 0;
+    c->launches = 0;
     c->initialised = true;
     return LBM_OK;
 }
@@ -772,6 +774,7 @@ lbm_status lbm_nd_step(lbm_nd *c, long n) {
         NDCK(c, nd_launch_pair(c, c->cur, c->stream));
         c->cur = 1 - c->cur;
         c->n += 2;
+        c->launches += 1;
     }
     if (left >= c->graph_chunk) {
         if (!c->graph[c->cur])
@@ -780,12 +783,14 @@ lbm_status lbm_nd_step(lbm_nd *c, long n) {
             NDCK(c, cudaGraphLaunch(c->graph[c->cur], c->stream));
             left -= c->graph_chunk;
             c->n += c->graph_chunk;
+            c->launches += c->graph_chunk;
         }
     }
     for (; left > 0; --left) {
         NDCK(c, nd_dispatch<StepNd>(c, c->cur, c->stream));
         c->cur = 1 - c->cur;
         c->n += 1;
+        c->launches += 1;
     }
     return LBM_OK;
 }
@@ -847,6 +852,8 @@ lbm_status lbm_nd_energy(lbm_nd *c, double *total) {
 }
 
 long lbm_nd_step_count(const lbm_nd *c) { return c ? c->n : -1; }
+
+long long lbm_nd_kernel_launches(const lbm_nd *c) { return c ? c->launches : -1; }
 
 const char *lbm_nd_last_error(const lbm_nd *c) {
     return c ? c->err.c_str() : g_nd_error.c_str();
