@@ -144,13 +144,19 @@ batch_kernel(const T *__restrict__ src, T *__restrict__ dst,
 // that the hardware hands the next item to whichever SM is free first: items
 // differ (an instance's last strip, its walls) and are two to three times the
 // resident warps, so a fixed share per block left the chip idle in the last
-// round (48 channels of 16 to 512 rows, 300 steps: 23.80 -> 23.08 ms).  The item count is read from device memory: captured
-// launches follow retirements.
+// round (48 channels of 16 to 512 rows, 300 steps: 23.80 -> 23.08 ms).  The
+// item count is read from device memory: captured launches follow retirements.
+// Blocks per SM by the register counts that were timed (us a step, 48 channels
+// of up to 512 rows, 64-row segments, without -> with): 15 at 4 steps (62.1 ->
+// 61.9; of up to 64 rows 11.3 -> 11.1), 12 at 5 (64.8 -> 65.1, up to 200 rows
+// 11.6 -> 10.9); 1 leaves the compiler the registers it asks for at 2 (102.8 ->
+// 99.6) and 3 steps (72.7 -> 70.9) and changes nothing at 6 and 7; at 8 steps
+// it made it spill 188 bytes (83.7 -> 88.1), so there is no bound there.
 constexpr int BW_WARPS = 1;        // one strip-segment per block, as the single-lattice kernel
 constexpr int BW_SMEM = BW_WARPS * wave::RING_ELEMS * (int)sizeof(float2);
 
 template <int K>
-__global__ void __launch_bounds__(BW_WARPS * 32, K == 4 ? 15 : K == 5 ? 12 : 1)
+__global__ void __launch_bounds__(BW_WARPS * 32, K == 4 ? 15 : K == 5 ? 12 : K == 8 ? 0 : 1)
 batch_wave(const float *__restrict__ src, float *__restrict__ dst,
            const InstDev<float> *__restrict__ inst, const WItem *__restrict__ items,
            const int *__restrict__ n_items, int halo, int seg_rows) {
