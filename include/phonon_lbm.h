@@ -339,15 +339,21 @@ lbm_status lbm_get_staged_config(const lbm_ctx *ctx, int *stages, int *ctas_per_
  * run this lattice (vector or scalar; staged with 2 or 3 stages and 8 or 4
  * consumer warps; cluster-resident; the multi-step kernel with 4, 5 or 6
  * steps per launch (2, 3 or 4 with 16-bit storage) and segments of 128 or
- * 256 rows, on lattices of at least 128 x 64 nodes), trial_steps steps each
- * (0 = 20) after 2 warm-up steps,
+ * 256 rows, on lattices of at least 128 x 64 nodes; what LBM_KERNEL_AUTO runs
+ * at this size: the multi-step kernel in a shape of its own, or the register
+ * tiles), trial_steps steps each (0 = 20) after 2 warm-up steps,
  * on the context's stream, and keeps the fastest for later lbm_step calls.
  * The timings run on the context's own buffers; when the context holds a
  * state (after lbm_init) both buffers are first copied to a temporary
  * device allocation (2 x lbm_population_bytes) and restored afterwards, so
  * the state and the step count are unchanged.  Outputs (may be NULL): the
  * chosen LBM_KERNEL_* and its mean time per step in microseconds.
- * Synchronous. */
+ * Another lattice takes the choice over with lbm_set_kernel(that kernel) and
+ * lbm_set_wave_config / lbm_set_staged_config of this one's shape.  The
+ * register tiles have no number of their own: where they win, `kernel` is
+ * that of their single steps, which lbm_set_kernel would select alone; a
+ * lattice of the same size left on LBM_KERNEL_AUTO (as lbm_create leaves it)
+ * runs them.  Synchronous. */
 lbm_status lbm_autotune(lbm_ctx *ctx, int trial_steps, int *kernel, double *us_per_step);
 
 /* Steps per captured CUDA graph chunk (even, >= 2), or 0 to launch every

@@ -468,7 +468,9 @@ class Lattice:
 
     def autotune(self, trial_steps: int = 20):
         """Pick the fastest kernel / staged shape for this lattice by timing
-        (state preserved); returns (kernel name, us per step)."""
+        (state preserved); returns (kernel name, us per step).  The name of the
+        single steps' kernel where the register tiles win: set_kernel with it
+        selects single steps, set_kernel("auto") the tiles."""
         k, us = ctypes.c_int(), ctypes.c_double()
         self._check(self._lib.lbm_autotune(self._ctx, int(trial_steps), ctypes.byref(k),
                                            ctypes.byref(us)))

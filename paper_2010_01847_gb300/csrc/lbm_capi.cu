@@ -1217,8 +1217,8 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
     if (trial_steps & 1) ++trial_steps;       // even: the buffers end where they began
     DeviceGuard g(c->device);
     if (lbm_status s = ensure_scratch(c, false)) return s;   // the status word
-    // wave: stages = steps, cw = segment rows; multi: the mid-size multi-step
-    // kernel the lattice's size picks, its single steps on `kernel`
+    // wave: stages = steps, cw = segment rows; multi: the register tiles, whose
+    // single steps are on `kernel`
     struct Cand { int kernel, stages, cw; bool multi; };
     Cand cands[17];
     int nc = 0;
@@ -1247,11 +1247,15 @@ lbm_status lbm_autotune(lbm_ctx *c, int trial_steps, int *kernel, double *us_per
     }
 
     for (int i = 0; i < nc; ++i) cands[i].multi = false;
+    // what a mid-size lattice runs untimed.  The strip march is LBM_KERNEL_WAVE
+    // with the plan's shape, so that a caller can give the choice to another
+    // lattice (lbm_get_kernel, lbm_get_wave_config); from 16 M nodes it is
+    // among the candidates above
     const Multi multi = plan_multi(c, cands[0].kernel);
-    // (from 16 M nodes the strip march is among the wave candidates)
-    if (multi.kind == MULTI_TILE ||
-        (multi.kind == MULTI_WAVE && (c->plane < WAVE_AUTO_NODES || c->nx < 256)))
+    if (multi.kind == MULTI_TILE)
         cands[nc++] = {cands[0].kernel, 0, 0, true};
+    else if (multi.kind == MULTI_WAVE && (c->plane < WAVE_AUTO_NODES || c->nx < 256))
+        cands[nc++] = {KERNEL_WAVE, multi.wave.steps, multi.wave.rows, false};
 
     // keep the state: copy both buffers aside when the lattice holds one
     void *saved = nullptr;
