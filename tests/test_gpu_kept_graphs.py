@@ -48,3 +48,44 @@ def test_selecting_the_default_again_after_other_steps_per_launch(precision, ste
     assert lat.step_count == plain.step_count
     for a, b in zip(lat.moments_device(), plain.moments_device()):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("precision,rounding", [
+    ("fp64", "nearest"), ("fp32", "nearest"), ("fp16", "nearest"), ("bf16", "stochastic")])
+def test_second_state_on_kept_graphs(precision, rounding):
+    """Single steps replayed from graphs of an earlier state: one of the same
+    amplitude, then one that moves the scale of 16-bit storage, which the
+    captured coefficients hold."""
+    nx, ny = 96, 65
+    make = lambda: plbm.Lattice(nx, ny, 0.9, 12.0, plbm.PERIODIC_GRADIENT, plbm.DIFFUSE_WALLS,
+                                1e-3, precision=precision, rounding=rounding, kernel="vector")
+    kept = make()
+    scales = []
+    for seed, amplitude in ((1, 1e-3), (2, 1e-3), (3, 0.25), (4, 0.25)):
+        f = start(nx, ny, seed, amplitude)
+        fresh = make()
+        for lat in (kept, fresh):
+            lat.init(*f)
+            lat.step(195)
+        assert kept.step_count == fresh.step_count == 195
+        assert np.array_equal(kept.populations(), fresh.populations())
+        scales.append(kept.storage_scale)
+    assert (scales[1] != scales[2]) == (precision in ("fp16", "bf16"))
+
+
+@pytest.mark.parametrize("lattice,shape,precision", [
+    (plbm.D3Q14, (12, 9, 15), "fp64"), (plbm.D3Q14, (16, 16, 16), "fp32"),
+    (plbm.D1Q2, (301,), "fp64")])
+def test_second_state_on_kept_graphs_nd(lattice, shape, precision):
+    rng = np.random.default_rng(5)
+    kept = plbm.LatticeND(lattice, shape, 0.9, 12.0, precision=precision)
+    for amplitude in (1e-3, 1e-3, 0.25):
+        e = 1.0 + amplitude * (rng.random(shape) - 0.5)
+        fresh = plbm.LatticeND(lattice, shape, 0.9, 12.0, precision=precision)
+        got = []
+        for lat in (kept, fresh):
+            lat.init(e)
+            lat.step(195)
+            got.append(lat.moments())
+        for a, b in zip(*got):
+            assert np.array_equal(a, b)
