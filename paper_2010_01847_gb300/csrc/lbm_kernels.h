@@ -197,7 +197,6 @@ cudaError_t launch_step_wave16(int precision, int steps, const void *src, void *
 // bit-identical to single steps; like the multi-step kernel it keeps the
 // post-collision state of the last step only.
 constexpr int TILE_MAX_WARPS = 16;
-constexpr int TILE_MAX_STEPS = 16;        // tiles of at least 32 own columns
 constexpr int TILE_MAX_ROWS = 4;
 constexpr long long TILE_MAX_NODES = 1LL << 28;     // 32-bit block counts and node columns
 struct TilePlan {
