@@ -646,9 +646,10 @@ def run_small(args):
     """The two small named workloads: the 128x32 phonon Poiseuille channel
     (10 000 steps, FP64 and FP32 storage) and the 4096x4 second-sound pulse
     (5 000 steps, Kn_R = 0.1, 1, 10, FP32).  Both are far too small to fill
-    the GPU: FP32 runs them cluster-resident (the whole lattice in one
-    cluster's shared memory, all steps in one launch), FP64 as
-    graph-captured launches, one per step.  The CPU-baseline leg (skipped
+    the GPU: FP32 runs the channel cluster-resident (the whole lattice in one
+    cluster's shared memory, all steps in one launch) and the pulse on register
+    tiles (several steps per launch; `kernel` then names that of the single
+    steps), FP64 as graph-captured launches, one per step.  The CPU-baseline leg (skipped
     with --no-cpu) runs the FP64 oracle on the same inputs, on all host
     cores: its time per step, and the GPU result's error against it (err_e,
     err_q as in the parity tests)."""
@@ -710,7 +711,8 @@ def run_small(args):
             "value": runs[1]["us_per_step"], "unit": "us/step", "n_gpus": 1,
             "higher_is_better": False, "dtype": "f32", "data": "synthetic",
             "config": {"workload": "poiseuille_128x32 (value: FP32) + second_sound_4096x4",
-                       "kernels": "FP32: cluster-resident, all steps in one launch; FP64: "
+                       "kernels": "FP32: cluster-resident, all steps in one launch (128x32); "
+                                  "register tiles, several steps per launch (4096x4); FP64: "
                                   "graph-captured launches"},
             "runs": runs, "gpu_launches": sum(r["gpu_launches"] for r in runs)}
     print(json.dumps(line), flush=True)

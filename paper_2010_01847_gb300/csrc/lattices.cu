@@ -148,7 +148,8 @@ step_nd(const T *src, T *dst, Dims g, CoefN<typename Store<T>::C> k) {
     chain_next();
     collide_nd<LAT>(d, k);
 #pragma unroll
-    for (int i = 0; i < Lat<LAT>::Q; ++i) __stcs(dst + (long long)i * g.plane + node, Store<T>::put(d[i]));
+    for (int i = 0; i < Lat<LAT>::Q; ++i)
+        __stcs(dst + (long long)i * g.plane + node, Store<T>::put(d[i]));
 }
 
 // Two time steps of an FP32 D3Q14 lattice per launch.  A single step is bound
@@ -161,11 +162,13 @@ step_nd(const T *src, T *dst, Dims g, CoefN<typename Store<T>::C> k) {
 // The next plane's loads are issued before step 2 of this one.  The
 // arithmetic is that of step_nd (pull_nd's values, collide_nd).
 // 192^3: 118.0 -> 83.9 us a step; 96^3 15.7 -> 14.4; below PAIR_MIN_NODES
-// chained single steps are faster (80^3 8.1 against 9.3 us, 64^3 4.8 against 7.2).  It reads and writes 787 MB of DRAM per launch
-// at 192^3, what two steps cannot do without; what is left is each plane's
+// chained single steps are faster (80^3 8.1 against 9.3 us, 64^3 4.8 against
+// 7.2).  At 192^3 a launch reads 426 MB of DRAM, 8 % more than the state, and
+// writes 352 MB before its end (the rest of the 396 MB is then in L2); DRAM is
+// busy 61 % of the time and the issue slots 66 %.  What is left is each plane's
 // barrier and loads, so several small blocks per SM do better than two large
 // ones: 32 x 16 threads and 2 blocks 95.9 us, 32 x 12 and 3 (spilling) 101.4,
-// 32 x 8 and 4 88.4, 32 x 10 and 3 83.9.
+// 32 x 8 and 4 88.4, 32 x 10 and 3 83.9 (64 registers, 4 bytes spilled).
 //
 // Shared memory: the 5 populations with c_z = +1 are pulled two positions
 // after they are written, those with c_z = 0 one, those with c_z = -1 in the

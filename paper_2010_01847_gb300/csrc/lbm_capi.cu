@@ -609,8 +609,9 @@ lbm_status init_from_device(lbm_ctx *c, const double *e, const double *qx, const
         }
     }
     // captured launches hold the coefficients, which depend on the scale only
-    // (capturing 64 steps again after every init took 0.2 ms: 512 x 128 FP64,
-    // 200 steps, 2100 -> 1891 us)
+    // (capturing 64 steps again after every init took 0.2 ms.  A pass of 512 x
+    // 128 FP64, 200 steps: 2094 us the first on a context, 1831 from the second
+    // on; launched step by step 2218 and 2112)
     if (c->scale != old_scale) drop_graphs(c);
     CK(c, dispatch<InitOp>(c, e, qx, qy));
     c->cur = 0;

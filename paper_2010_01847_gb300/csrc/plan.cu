@@ -13,7 +13,11 @@ namespace plbm {
 // costs 3900 plus 85 per row a block holds (the loads and stores of 64
 // columns of 8 planes), a step 240 (barrier and the dependency chain of one
 // row) plus 115 issue cycles per row of the busiest scheduler.  Blocks of one
-// SM share its schedulers.
+// SM share its schedulers.  No sweep had sides along x and y, and the estimate
+// has no term for their rules: 0.74 us a step for the 201 x 201 square, which
+// takes 1.38; there it orders the plans as if the lattice were a channel.  The
+// registers per thread that limit the blocks of an SM are rounded up over the
+// boundary kinds: 56 to 78 at R = 1, 89 to 118 at R = 2, 123 to 128 above.
 double tile_plan(int nx, int ny, int bc_x, int bc_y, int sms, TilePlan *out) {
     const bool open_x = bc_x == BC_SIDES, open_y = bc_y == BC_SIDES || bc_y == BC_WALLS;
     double best = 0.0;

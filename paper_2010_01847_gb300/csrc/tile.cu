@@ -6,7 +6,8 @@
 // its own: one launch per step costs 2-4 us whatever it does.  Here the
 // lattice is cut into about one tile per SM: 64 columns (two adjacent nodes
 // per lane) by as many rows as the block's warps hold, R rows per warp, all
-// 8 planes of every node in registers.  A block loads its tile and a halo,
+// 8 planes of every node in registers (at R = 4 the compiler keeps 32 to 60
+// bytes of a thread's 128-register state in local memory).  A block loads its tile and a halo,
 // advances it K steps and writes the tile's own nodes; the outermost ring of
 // the halo goes wrong one node per step.  Within a warp the c_y neighbours
 // are the thread's other rows and the c_x neighbours come from the lane's
@@ -19,7 +20,7 @@
 // so any nx, ny and boundary kind runs here; beyond a wall or side the tile
 // computes values that the treatments of Section 2.5 replace wherever a valid
 // node would pull them.  The arithmetic is that of every FP32 kernel
-// (collide_f32 on node pairs, the same operations in the same order), so the
+// (collide_f32 node by node, the same operations in the same order), so the
 // results are bit-identical to single steps.
 //
 // Launches are chained with programmatic dependent launch: the next launch
